@@ -225,7 +225,7 @@ int xshare_moe_forward(const uint16_t *x, const float *W_g, const uint16_t *W_ga
  * device).  Neither can hand xshare_route a workspace.
  *
  * Same arguments and results as xshare_route, minus the workspace.  The
- * scratch is a fixed array inside the library's device code (about 420 KB
+ * scratch is a fixed array inside the library's device code (about 350 KB
  * on every GPU that loads the library, held until the process exits), so:
  *   - B is limited to 1024 tokens (N <= 1024 and k <= 16 as elsewhere); a
  *     larger B returns XS_ERR_SHAPE and launches nothing;

@@ -91,7 +91,6 @@ RouteArgs route_args(const Plan &pl, void *ws, int B, int N, int k, int budget, 
   a.toptok = at<int32_t>(ws, pl.toptok);
   a.counts = at<int32_t>(ws, pl.counts);
   a.offsets = at<int32_t>(ws, pl.offsets);
-  a.perm = at<int32_t>(ws, pl.perm);
   a.pos = at<int32_t>(ws, pl.pos);
   a.tiles = at<Tile>(ws, pl.tiles);
   a.meta = at<Meta>(ws, pl.meta);
@@ -126,7 +125,6 @@ Plan make_plan(int B, int N, int k, int d, int F, bool with_ffn, int n_sms, int 
   pl.toptok = take((size_t)B * kMaxK * 4);
   pl.counts = take((size_t)N * 4);
   pl.offsets = take((size_t)(N + 1) * 4);
-  pl.perm = take((size_t)B * k * 4);
   pl.pos = take((size_t)B * k * 4);
   pl.tiles = take((size_t)pl.max_tiles * sizeof(Tile));
   pl.meta = take(sizeof(Meta));
@@ -331,8 +329,8 @@ int xs::forward_impl(const FwdCall &c, FwdStep step) {
     // a longer window before the gate/up kernel: twice the warm-up.
     pf.pf_bytes = (B + kChunk - 1) / kChunk > kFuseChunks ? 2 * kGatherPrefetchBytes : kGatherPrefetchBytes;
   }
-  if (launch_gather(c.x, a.perm, a.meta, const_cast<uint16_t *>(f.xp), ep ? f.out : nullptr,
-                    pl.max_rows, B, d, k, pf, s) != cudaSuccess ||
+  if (launch_gather(c.x, a, const_cast<uint16_t *>(f.xp), ep ? f.out : nullptr, d, sms, pf, s) !=
+          cudaSuccess ||
       !mark(4))
     return XS_ERR_CUDA;
   if (launch_ffn_gate_up(f, s) != cudaSuccess || !mark(5)) return XS_ERR_CUDA;

@@ -309,9 +309,9 @@ __device__ __forceinline__ void block_scan3(int (&v)[3], int (&tot)[3], int *s_t
 //       closed form).  CTAs C .. 2C - 1 rank every token's top-k over E at
 //       the same time and count the plain top-k union (a statistic).
 //   refine_kernel (a6, a7): per token the top-k' inside S with renormalised
-//       weights.  The CTA that finishes last counts the pairs per expert,
-//       takes the prefix sums, writes the FFN tiles and scatters the pairs
-//       stably by expert.
+//       weights, and the chunk's pairs per expert.  The CTA that finishes
+//       last takes the prefix sums over chunks and experts and writes the
+//       FFN tiles; the pairs are placed by the kernel after it.
 //
 // "Last to finish" uses an arrival counter per group of CTAs (done[0] the
 // selection, done[1] the refinement, done[2] the union), cleared before the
@@ -460,177 +460,161 @@ __device__ __forceinline__ void refine_tokens(const RouteArgs &a, const uint8_t 
   }
 }
 
-struct PermSmem {
-  int32_t *counts, *cursor, *chunk, *tmp, *scal, *wcnt;  // wcnt: [32][N] (N <= kScatterMaxN)
-  const int32_t *ids;  // nullable: the ids in shared memory (else read from global)
-};
+// FFN tiles of expert e's run of cnt rows from row0, as tiles[tile0 ...].
+// tile_count() says how many.
+__device__ __forceinline__ int tile_count(int cnt) { return (cnt + kTileTok - 1) / kTileTok; }
 
-// Counting sort of all pairs by expert, stable in (token, slot) (a7), the FFN
-// tiles and the statistics.  One CTA, once every token's ids are written and
-// visible; the meta block already holds the selection's fields.
-__device__ void build_permutation(const RouteArgs &a, PermSmem sm) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int nwarps = blockDim.x >> 5;
-  const int B = a.B, N = a.N, k = a.k;
-  const int P = B * k;
-  for (int j = tid; j < N; j += blockDim.x) sm.counts[j] = 0;
-  __syncthreads();
-  for (int q = tid; q < P; q += blockDim.x) {
-    const int e = sm.ids ? sm.ids[q] : __ldcg(a.ids + q);
-    if ((unsigned)e < (unsigned)N) atomicAdd(&sm.counts[e], 1);
+__device__ __forceinline__ void write_tiles(Tile *tiles, int tile0, int e, int row0, int cnt) {
+  for (int tt = 0; tt * kTileTok < cnt; ++tt) {
+    Tile tl;
+    tl.expert = e;
+    tl.row0 = row0 + tt * kTileTok;
+    tl.ntok = min(kTileTok, cnt - tt * kTileTok);
+    tl.pad = 0;
+    tiles[tile0 + tt] = tl;
+  }
+}
+
+// The counting sort of all pairs by expert, stable in (token, slot) (a7), for
+// more than kFuseChunks chunks.  A token uses an expert in at most one slot,
+// so a pair's row is
+//   first row of its expert + the expert's tokens in the chunks before
+//   + its rank among the expert's tokens of its own chunk.
+// Every refinement CTA knows the rank and the counts of its own chunk
+// (publish_chunk); the last one to finish turns the counts into first rows
+// per chunk and expert (build_offsets); the pairs are then placed by the
+// kernel that comes next and has the whole GPU: the gather kernel, or
+// scatter_kernel when only the routing was asked for.  Until then pos[q]
+// holds the rank.  Before, one CTA scattered every pair itself, bound by its
+// latency (six barriers per 1024 pairs, one warp alone for N > 256); whole
+// calls on GB300: routing B = 2048, N = 256 77.0 -> 29.9 us, layer forward
+// B = 2048, N = 128 (16384 pairs) 471 -> 423 us, B = 8192, N = 64 (65536
+// pairs) 1691 -> 1479 us (the last two with the gather reading a token once
+// for several rows), B = 256 unchanged (219.5 us).
+//
+// The counts are uint8 (a chunk has 32 tokens) in chunk_marks, the first
+// rows int32 in chunk_col: both regions are free once the selection is done.
+
+// pos[q] = rank and the chunk's counts from the chunk's ids (ids_s, t-major);
+// s_tm: [N] token masks, zero on entry.
+__device__ __forceinline__ void publish_chunk(const RouteArgs &a, const int32_t *ids_s, uint32_t *s_tm,
+                                              int c, int nt) {
+  const int N = a.N, k = a.k, q0 = c * kChunk * k;
+  for (int i = threadIdx.x; i < nt * k; i += blockDim.x) {
+    const int e = ids_s[i];
+    if ((unsigned)e < (unsigned)N) atomicOr(&s_tm[e], 1u << (i / k));
   }
   __syncthreads();
+  for (int i = threadIdx.x; i < nt * k; i += blockDim.x) {
+    const int e = ids_s[i];
+    a.pos[q0 + i] = (unsigned)e < (unsigned)N ? __popc(s_tm[e] & ((1u << (i / k)) - 1u)) : -1;
+  }
+  uint8_t *cnt = a.chunk_marks + (size_t)c * 2 * N;
+  for (int j = threadIdx.x; j < N; j += blockDim.x) cnt[j] = static_cast<uint8_t>(__popc(s_tm[j]));
+}
+
+// One CTA, once every chunk is published and visible: counts, offsets, tiles,
+// statistics and the first row of every (chunk, expert).  The meta block
+// already holds the selection's fields.  s_part, s_off: [kRouteThreads]
+// scratch, s_tmp: [200].  The chunks are split over blockDim / N parts, so
+// that each thread adds a short run of them.
+__device__ void build_offsets(const RouteArgs &a, int32_t *s_part, int32_t *s_off, int32_t *s_tmp) {
+  const int tid = threadIdx.x;
+  const int B = a.B, N = a.N;
+  const int C = chunk_count(B);
+  const int Np = (N + 31) & ~31, parts = blockDim.x / Np;
+  const int e = tid % Np, part = tid / Np;
+  const int per = (C + parts - 1) / parts;
+  const int c_lo = min(part * per, C), c_hi = part < parts ? min(c_lo + per, C) : c_lo;
+  const uint8_t *cnt = a.chunk_marks + e;
+  int sum = 0;
+  if (e < N) {
+#pragma unroll 16
+    for (int c = c_lo; c < c_hi; ++c) sum += __ldcg(cnt + (size_t)c * 2 * N);
+  }
+  if (part < parts) s_part[part * Np + e] = sum;
+  __syncthreads();
+  int n_e = 0;
+  if (tid < N)
+    for (int q = 0; q < parts; ++q) {  // exclusive over the parts, and the expert's total
+      const int x = s_part[q * Np + tid];
+      s_part[q * Np + tid] = n_e;
+      n_e += x;
+    }
+  int v[3] = {n_e, tile_count(n_e), n_e > 0 ? 1 : 0}, tot[3];
+  block_scan3(v, tot, s_tmp);
+  if (tid < N) {
+    s_off[tid] = v[0];
+    a.counts[tid] = n_e;
+    a.offsets[tid] = v[0];
+    if (a.counts_out) a.counts_out[tid] = n_e;
+    if (a.offsets_out) a.offsets_out[tid] = v[0];
+    write_tiles(a.tiles, v[1], tid, v[0], n_e);
+  }
+  // This call's FFN work (Sec. 5): the tiles and rows of the experts of
+  // group ep_rank, a contiguous index range, hence contiguous tiles and
+  // rows; shared experts go to rank 0.  Without expert parallelism: all.
   {
-    const int cnt = tid < N ? sm.counts[tid] : 0;
-    int v[3] = {cnt, (cnt + kTileTok - 1) / kTileTok, cnt > 0 ? 1 : 0}, tot[3];
-    block_scan3(v, tot, sm.tmp);
-    if (tid < N) {
-      sm.cursor[tid] = v[0];
-      a.counts[tid] = cnt;
-      a.offsets[tid] = v[0];
-      if (a.counts_out) a.counts_out[tid] = cnt;
-      if (a.offsets_out) a.offsets_out[tid] = v[0];
-      for (int tt = 0; tt * kTileTok < cnt; ++tt) {
-        Tile tl;
-        tl.expert = tid;
-        tl.row0 = v[0] + tt * kTileTok;
-        tl.ntok = min(kTileTok, cnt - tt * kTileTok);
-        tl.pad = 0;
-        a.tiles[v[1] + tt] = tl;
-      }
+    const int G = a.ep_ranks > 1 ? a.ep_ranks : 1, g = G > 1 ? a.ep_rank : 0;
+    const int e_lo = g * (N / G), e_hi = (g + 1) * (N / G);
+    Meta *m = a.meta;
+    if (tid == e_lo) {
+      m->ffn_t0 = v[1];
+      m->row0 = v[0];
+    }
+    if (e_hi < N && tid == e_hi) {
+      m->ffn_t1 = v[1];
+      m->row1 = v[0];
     }
     if (tid == 0) {
       a.offsets[N] = tot[0];
       if (a.offsets_out) a.offsets_out[N] = tot[0];
-      sm.scal[1] = tot[0];  // pairs
-      sm.scal[2] = tot[1];  // tiles
-      sm.scal[3] = tot[2];  // used experts
-    }
-    // This call's FFN work (Sec. 5): the tiles and rows of the experts of
-    // group ep_rank, a contiguous index range, hence contiguous tiles and
-    // rows; shared experts go to rank 0.  Without expert parallelism: all.
-    {
-      const int G = a.ep_ranks > 1 ? a.ep_ranks : 1, g = G > 1 ? a.ep_rank : 0;
-      const int e_lo = g * (N / G), e_hi = (g + 1) * (N / G);
-      Meta *m = a.meta;
-      if (tid == e_lo) {
-        m->ffn_t0 = v[1];
-        m->row0 = v[0];
+      if (e_hi >= N) {
+        m->ffn_t1 = tot[1];
+        m->row1 = tot[0];
       }
-      if (e_hi < N && tid == e_hi) {
-        m->ffn_t1 = v[1];
-        m->row1 = v[0];
+      const int own_shared = g == 0 ? 1 : 0, shared_tiles = a.n_shared * tile_count(B);
+      m->ffn_s0 = tot[1];
+      m->ffn_s1 = tot[1] + own_shared * shared_tiles;
+      m->srows = own_shared;
+      // Field by field: union_topk belongs to the union CTAs (score_kernel).
+      m->n_pairs = tot[0];  // == B * kp unless scores were non-finite
+      m->n_tiles = tot[1] + shared_tiles;
+      m->n_used = tot[2];
+      m->n_rows = tot[0] + a.n_shared * B;
+      if (a.stats) {
+        xs_stats *st = a.stats;
+        st->n_selected = m->n_selected;
+        st->n_used = tot[2];
+        st->max_group_load = m->max_group_load;
+        st->n_pairs = tot[0];
+        st->status = m->status;
+        st->reserved[0] = st->reserved[1] = 0;
       }
-      if (tid == 0) {
-        if (e_hi >= N) {
-          m->ffn_t1 = tot[1];
-          m->row1 = tot[0];
-        }
-        const int own_shared = g == 0 ? 1 : 0;
-        m->ffn_s0 = tot[1];
-        m->ffn_s1 = tot[1] + own_shared * a.n_shared * ((B + kTileTok - 1) / kTileTok);
-        m->srows = own_shared;
-      }
-    }
-    // Shared experts: every token, in token order, after the routed pairs.
-    const int tpt = (B + kTileTok - 1) / kTileTok;
-    for (int i = tid; i < a.n_shared * tpt; i += blockDim.x) {
-      const int j = i / tpt, tt = i - j * tpt;
-      Tile tl;
-      tl.expert = N + j;
-      tl.row0 = tot[0] + j * B + tt * kTileTok;
-      tl.ntok = min(kTileTok, B - tt * kTileTok);
-      tl.pad = 0;
-      a.tiles[tot[1] + i] = tl;
     }
   }
+  // Shared experts: every token, in token order, after the routed pairs.
+  for (int j = tid; j < a.n_shared; j += blockDim.x)
+    write_tiles(a.tiles, tot[1] + j * tile_count(B), N + j, tot[0] + j * B, B);
   __syncthreads();
-  const unsigned lt = (1u << lane) - 1u;
-  if (N <= kScatterMaxN) {
-    // Chunks of blockDim pairs: rank inside a warp by match_any, then an
-    // exclusive prefix over the warps of the chunk for every expert.
-    for (int base = 0; base < P; base += blockDim.x) {
-      // Only the warps that hold pairs of this chunk count.
-      const int nw_used = min(nwarps, (P - base + 31) / 32);
-      for (int i = tid; i < nw_used * N; i += blockDim.x) sm.wcnt[i] = 0;
-      const int q = base + tid;
-      int e = (q < P) ? (sm.ids ? sm.ids[q] : __ldcg(a.ids + q)) : -1;
-      if ((unsigned)e >= (unsigned)N) e = -1;
-      const unsigned peers = __match_any_sync(kFull, e);
-      const int rank = __popc(peers & lt);
-      __syncthreads();
-      if (e >= 0 && rank == 0) sm.wcnt[warp * N + e] = __popc(peers);
-      __syncthreads();
-      if (tid < N) {
-        int run = 0;
-        for (int w = 0; w < nw_used; ++w) {
-          const int x = sm.wcnt[w * N + tid];
-          sm.wcnt[w * N + tid] = run;
-          run += x;
-        }
-        sm.chunk[tid] = run;
-      }
-      __syncthreads();
-      if (e >= 0) {
-        const int r = sm.cursor[e] + sm.wcnt[warp * N + e] + rank;
-        a.perm[r] = q;
-        a.pos[q] = r;
-        if (a.perm_out) a.perm_out[r] = q;
-      } else if (q < P) {
-        a.pos[q] = -1;
-      }
-      __syncthreads();
-      if (tid < N) sm.cursor[tid] += sm.chunk[tid];
-      __syncthreads();
-    }
-  } else if (warp == 0) {
-    for (int base = 0; base < P; base += 32) {
-      const int q = base + lane;
-      int e = (q < P) ? (sm.ids ? sm.ids[q] : __ldcg(a.ids + q)) : -1;
-      if ((unsigned)e >= (unsigned)N) e = -1;
-      const unsigned peers = __match_any_sync(kFull, e);
-      const int rank = __popc(peers & lt);
-      const int old = (e >= 0) ? sm.cursor[e] : 0;
-      __syncwarp();
-      if (e >= 0) {
-        const int r = old + rank;
-        a.perm[r] = q;
-        a.pos[q] = r;
-        if (a.perm_out) a.perm_out[r] = q;
-        if (rank == 0) sm.cursor[e] = old + __popc(peers);
-      } else if (q < P) {
-        a.pos[q] = -1;
-      }
-      __syncwarp();
-    }
-  }
-  if (tid == 0) {
-    // Field by field: union_topk belongs to the union CTAs (score_kernel).
-    Meta *m = a.meta;
-    m->n_pairs = sm.scal[1];  // == B * kp unless scores were non-finite
-    m->n_tiles = sm.scal[2] + a.n_shared * ((B + kTileTok - 1) / kTileTok);
-    m->n_used = sm.scal[3];
-    m->n_rows = sm.scal[1] + a.n_shared * B;
-    if (a.stats) {
-      xs_stats *st = a.stats;
-      st->n_selected = m->n_selected;
-      st->n_used = sm.scal[3];
-      st->max_group_load = m->max_group_load;
-      st->n_pairs = sm.scal[1];
-      st->status = m->status;
-      st->reserved[0] = st->reserved[1] = 0;
+  if (e < N && part < parts) {
+    int run = s_off[e] + s_part[part * Np + e];
+    int32_t *first = reinterpret_cast<int32_t *>(a.chunk_col) + e;
+#pragma unroll 16
+    for (int c = c_lo; c < c_hi; ++c) {
+      const int x = __ldcg(cnt + (size_t)c * 2 * N);
+      first[(size_t)c * N] = run;
+      run += x;
     }
   }
 }
 
-// The same permutation, tiles and statistics as build_permutation, for a
-// batch of at most 64 tokens, with two block barriers instead of about ten.
-// A pair's position in its expert's run is the number of earlier tokens
-// routed to that expert (a token uses an expert in at most one slot), so one
-// 32-bit token mask per expert and 32-token chunk gives the counts and every
-// position.  The masks (sm.cursor for tokens 0-31, sm.counts for 32-63, as
-// uint32) must be zero on entry.  ids: ids_s[t * k + s] in shared memory
-// (one chunk), else the ids in global memory.
+// The same permutation, tiles and statistics for a batch of at most 64
+// tokens, in one CTA with two block barriers: one 32-bit token mask per
+// expert and 32-token chunk gives the counts and every position.  The masks
+// (s_tm0 for tokens 0-31, s_tm1 for 32-63; [N] each) must be zero on entry;
+// s_off: [N] scratch.  ids: ids_s[t * k + s] in shared memory (one chunk),
+// else the ids in global memory.
 //   1. every pair (t, s): mask[t / 32][e] |= 1 << (t % 32) (shared-memory
 //      atomic).
 //   2. warp 0, 32 experts per round: counts, exclusive prefix over the
@@ -638,13 +622,11 @@ __device__ void build_permutation(const RouteArgs &a, PermSmem sm) {
 //      tile), tiles, meta.
 //   3. warp t, lane s < k: position of pair (t, s) = offset[e] + the tokens
 //      of e in the chunks before + popc(mask[t / 32][e] & (tokens below t)).
-__device__ void build_permutation_small(const RouteArgs &a, PermSmem sm, const int32_t *ids_s) {
+__device__ void build_permutation_small(const RouteArgs &a, uint32_t *s_tm0, uint32_t *s_tm1,
+                                        int32_t *s_off, const int32_t *ids_s) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nwarps = blockDim.x >> 5;
   const int B = a.B, N = a.N, k = a.k;
-  uint32_t *s_tm0 = reinterpret_cast<uint32_t *>(sm.cursor);  // [N] tokens 0-31 per expert
-  uint32_t *s_tm1 = reinterpret_cast<uint32_t *>(sm.counts);  // [N] tokens 32-63 per expert
-  int32_t *s_off = sm.chunk;                                   // [N] first row per expert
   auto id_of = [&](int q) { return ids_s != nullptr ? ids_s[q] : __ldcg(a.ids + q); };
   for (int q = tid; q < B * k; q += blockDim.x) {
     const int e = id_of(q), t = q / k;
@@ -745,7 +727,6 @@ __device__ void build_permutation_small(const RouteArgs &a, PermSmem sm, const i
         const uint32_t below = (1u << (t & 31)) - 1u;
         const int r = s_off[e] + (t < 32 ? __popc(s_tm0[e] & below)
                                          : __popc(s_tm0[e]) + __popc(s_tm1[e] & below));
-        a.perm[r] = q;
         a.pos[q] = r;
         if (a.perm_out) a.perm_out[r] = q;
       } else {
@@ -866,8 +847,8 @@ __global__ void __launch_bounds__(kRouteThreads, 1) score_kernel(RouteArgs a) {
   __shared__ int32_t s_gl[kMaxN + 1];
   __shared__ int32_t s_top[kChunk][kMaxK];
   __shared__ int32_t s_scal[4];
-  __shared__ int32_t s_counts[kMaxN];   // permutation, when it runs in this kernel
-  __shared__ int32_t s_cursor[kMaxN];
+  __shared__ uint32_t s_counts[kMaxN];  // token masks of the permutation, when it runs in
+  __shared__ uint32_t s_cursor[kMaxN];  // this kernel: tokens 32-63, tokens 0-31
   __shared__ int32_t s_chunk[kMaxN];
   __shared__ int32_t s_tmp[200];
   __shared__ int s_rflag;               // a router CTA reported a timeout
@@ -1214,19 +1195,17 @@ __global__ void __launch_bounds__(kRouteThreads, 1) score_kernel(RouteArgs a) {
   if (C > 1) __threadfence();
   __syncthreads();
   static_assert(kFuseChunks <= 2, "the fused permutation takes at most two 32-token chunks");
-  build_permutation_small(a, PermSmem{s_counts, s_cursor, s_chunk, s_tmp, s_scal, nullptr, nullptr},
-                          ids_s);
+  build_permutation_small(a, s_cursor, s_counts, s_chunk, ids_s);
 }
 
 template <int kQ>
 __global__ void __launch_bounds__(kRouteThreads, 1) refine_kernel(RouteArgs a) {
-  extern __shared__ int32_t s_wcnt[];   // [32][N] per-warp counts of the scatter (N <= 256)
   __shared__ uint8_t s_mask[kMaxN];
-  __shared__ int32_t s_counts[kMaxN];
-  __shared__ int32_t s_cursor[kMaxN];
+  __shared__ uint32_t s_tm[kMaxN];      // token masks of the chunk, then build_offsets scratch
   __shared__ int32_t s_chunk[kMaxN];
+  __shared__ int32_t s_ids[kChunk * kMaxK];
   __shared__ int32_t s_tmp[200];
-  __shared__ int32_t s_scal[4];
+  __shared__ int32_t s_last;
 
   pdl_wait();
   pdl_trigger();
@@ -1235,19 +1214,45 @@ __global__ void __launch_bounds__(kRouteThreads, 1) refine_kernel(RouteArgs a) {
   const int C = chunk_count(B), c = blockIdx.x;
   const int t0 = c * kChunk, nt = min(kChunk, B - t0);
   const int kp = a.meta->kprime;
-  for (int j = tid; j < N; j += blockDim.x) s_mask[j] = a.mask[j];
+  for (int j = tid; j < N; j += blockDim.x) {
+    s_mask[j] = a.mask[j];
+    s_tm[j] = 0u;
+  }
   __syncthreads();
   refine_tokens<kQ>(a, s_mask, a.meta->n_selected, s_chunk, s_tmp, t0, t0 + nt, kp,
-                    [&](int t) { return a.p + (size_t)t * N; });
+                    [&](int t) { return a.p + (size_t)t * N; }, s_ids);
+  __syncthreads();
+  publish_chunk(a, s_ids, s_tm, c, nt);
 
-  // ---- the last CTA to finish builds the permutation (a7) ----
+  // ---- the last CTA to finish places the chunks (a7) ----
   __threadfence();
   __syncthreads();
-  if (tid == 0) s_scal[0] = (atomicAdd(&a.done[1], 1) == C - 1) ? 1 : 0;
+  if (tid == 0) s_last = (atomicAdd(&a.done[1], 1) == C - 1) ? 1 : 0;
   __syncthreads();
-  if (!s_scal[0]) return;
+  if (!s_last) return;
   __threadfence();
-  build_permutation(a, PermSmem{s_counts, s_cursor, s_chunk, s_tmp, s_scal, s_wcnt, nullptr});
+  build_offsets(a, reinterpret_cast<int32_t *>(s_tm), s_chunk, s_tmp);
+}
+
+// Row of pair q = t * k + s: final in pos[q] for up to kFuseChunks chunks
+// (first == nullptr), else its rank plus the first row of (chunk, expert).
+__device__ __forceinline__ int pair_row(const int32_t *ids, const int32_t *pos, const int32_t *first,
+                                        int N, int q, int t) {
+  const int r = pos[q];
+  return r < 0 || first == nullptr ? r : r + first[(size_t)(t / kChunk) * N + ids[q]];
+}
+
+// The permutation of a routing call (no gather follows).
+__global__ void __launch_bounds__(256) scatter_kernel(const int32_t *__restrict__ ids,
+                                                      const int32_t *__restrict__ pos,
+                                                      const int32_t *__restrict__ first,
+                                                      int32_t *__restrict__ perm, int P, int N, int k) {
+  pdl_wait();
+  pdl_trigger();
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= P) return;
+  const int r = pair_row(ids, pos, first, N, q, q / k);
+  if (r >= 0) perm[r] = q;
 }
 
 // ---- a1: router logits h = W_g x, fp32.
@@ -1425,37 +1430,65 @@ __device__ void warm_gate_up(const GatherPf &g, int32_t *s_sel, int *s_n) {
   }
 }
 
-// Xp[row] = x[token of pair perm[row]], 16-byte vectors, for the rows this
-// call's FFN computes; with expert parallelism the other rows of zero_out
-// (computed by other ranks) are set to zero instead.  Before that (packed
-// weights), the gate/up kernel's first weights are brought into L2 as soon
-// as the selected set is published.
+// Places the pairs (pos[q] = row) and copies their tokens: Xp[row] = x[t],
+// 16-byte vectors, for the rows this call's FFN computes; with expert
+// parallelism the other rows of zero_out (computed by other ranks) are set
+// to zero instead.  Before that (packed weights), the gate/up kernel's first
+// weights are brought into L2 as soon as the selected set is published.
+//
+// A block takes per_block consecutive slots of one token (slots k ..
+// k + n_shared - 1 are the shared experts' rows) and reads the token once for
+// all of them.
+constexpr int kGatherSlots = kMaxK + kMaxShared;
+
 __global__ void __launch_bounds__(256) gather_kernel(const uint16_t *__restrict__ x,
-                                                     const int32_t *__restrict__ perm,
+                                                     const int32_t *__restrict__ ids, int32_t *pos,
+                                                     const int32_t *__restrict__ first,
                                                      const Meta *__restrict__ meta,
                                                      uint16_t *__restrict__ xp,
-                                                     float *__restrict__ zero_out, int B, int d,
-                                                     int k, GatherPf pf) {
+                                                     float *__restrict__ zero_out, int B, int N,
+                                                     int d, int k, int n_shared, int per_block,
+                                                     GatherPf pf) {
   __shared__ int32_t s_sel[kMaxN];
   __shared__ int s_n;
+  __shared__ int32_t s_row[kGatherSlots];   // row of each slot; ~row if another rank computes it
   if (pf.pk != nullptr && static_cast<int>(blockIdx.x) < kGatherWarmBlocks) warm_gate_up(pf, s_sel, &s_n);
   pdl_wait();
   pdl_trigger();
-  const int row = blockIdx.x;
-  const int P = meta->n_pairs;
-  if (row >= meta->n_rows) return;
-  const bool mine = row < P ? (row >= meta->row0 && row < meta->row1) : meta->srows != 0;
-  if (!mine) {
-    if (zero_out != nullptr) {
-      float4 *dst = reinterpret_cast<float4 *>(zero_out + static_cast<size_t>(row) * d);
+  const int slots = k + n_shared, groups = (slots + per_block - 1) / per_block;
+  const int t = blockIdx.x / groups, s0 = (blockIdx.x - t * groups) * per_block;
+  const int n = min(per_block, slots - s0);
+  if (static_cast<int>(threadIdx.x) < n) {
+    const int s = s0 + threadIdx.x, q = t * k + s;
+    int row;
+    bool mine;
+    if (s < k) {
+      row = pair_row(ids, pos, first, N, q, t);
+      if (first != nullptr) pos[q] = row;
+      mine = row >= meta->row0 && row < meta->row1;
+      if (row < 0) row = INT_MIN;  // unrouted slot: no row
+    } else {
+      row = meta->n_pairs + (s - k) * B + t;
+      mine = meta->srows != 0;
+    }
+    s_row[threadIdx.x] = mine || row == INT_MIN ? row : ~row;
+  }
+  __syncthreads();
+  const uint4 *src = reinterpret_cast<const uint4 *>(x + (size_t)t * d);
+  for (int i = threadIdx.x; i < d / 8; i += blockDim.x) {
+    const uint4 v = __ldg(src + i);
+    for (int s = 0; s < n; ++s) {
+      const int row = s_row[s];
+      if (row >= 0) reinterpret_cast<uint4 *>(xp + (size_t)row * d)[i] = v;
+    }
+  }
+  if (zero_out != nullptr)
+    for (int s = 0; s < n; ++s) {
+      const int row = s_row[s];
+      if (row >= 0 || row == INT_MIN) continue;
+      float4 *dst = reinterpret_cast<float4 *>(zero_out + static_cast<size_t>(~row) * d);
       for (int i = threadIdx.x; i < d / 4; i += blockDim.x) dst[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    return;
-  }
-  const int t = row < P ? perm[row] / k : (row - P) % B;  // routed pair, else shared row
-  const uint4 *src = reinterpret_cast<const uint4 *>(x + (size_t)t * d);
-  uint4 *dst = reinterpret_cast<uint4 *>(xp + (size_t)row * d);
-  for (int i = threadIdx.x; i < d / 8; i += blockDim.x) dst[i] = __ldg(src + i);
 }
 
 // ---- a9: y_t = [x_t +] sum over slots s < k' of w_ts * out[pos(t, s)]
@@ -1532,8 +1565,7 @@ cudaError_t launch_route_q(const RouteArgs &a, cudaStream_t s) {
   const int C = (a.B + kChunk - 1) / kChunk;
   RouteArgs b = a;
   b.fuse_refine = C <= kFuseChunks ? 1 : 0;
-  const int wcnt = a.N <= kScatterMaxN ? 32 * a.N * 4 : 0;
-  const int dyn1 = kChunk * a.N * 4 + (b.fuse_refine ? wcnt : 0);
+  const int dyn1 = kChunk * a.N * 4;
   cudaError_t e = cudaFuncSetAttribute(score_kernel<kQ>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, dyn1);
   if (e != cudaSuccess) return e;
@@ -1547,9 +1579,11 @@ cudaError_t launch_route_q(const RouteArgs &a, cudaStream_t s) {
     e = cudaEventRecord(reinterpret_cast<cudaEvent_t>(a.events[0]), s);
     if (e != cudaSuccess) return e;
   }
-  e = cudaFuncSetAttribute(refine_kernel<kQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, wcnt);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(refine_kernel<kQ>, dim3(C), dim3(kRouteThreads), (size_t)wcnt, s, b);
+  e = launch_pdl(refine_kernel<kQ>, dim3(C), dim3(kRouteThreads), 0, s, b);
+  if (e != cudaSuccess || a.perm_out == nullptr) return e;
+  const int P = a.B * a.k;
+  return launch_pdl(scatter_kernel, dim3((P + 255) / 256), dim3(256), 0, s, a.ids, a.pos,
+                    reinterpret_cast<const int32_t *>(a.chunk_col), a.perm_out, P, a.N, a.k);
 }
 
 cudaError_t launch_route(const RouteArgs &a, cudaStream_t s) {
@@ -1566,11 +1600,18 @@ cudaError_t launch_router_logits(const uint16_t *x, const float *Wg, float *h, i
                     done);
 }
 
-cudaError_t launch_gather(const uint16_t *x, const int32_t *perm, const Meta *meta,
-                          uint16_t *xp, float *zero_out, int max_rows, int B, int d, int k,
-                          const GatherPf &pf, cudaStream_t s) {
-  return launch_pdl(gather_kernel, dim3(max_rows), dim3(256), 0, s, x, perm, meta, xp, zero_out, B,
-                    d, k, pf);
+cudaError_t launch_gather(const uint16_t *x, const RouteArgs &a, uint16_t *xp, float *zero_out, int d,
+                          int n_sms, const GatherPf &pf, cudaStream_t s) {
+  // One slot per block until that would be more than eight blocks per SM.
+  const int slots = a.k + a.n_shared;
+  int per_block = static_cast<int>(static_cast<long long>(a.B) * slots / (8 * n_sms));
+  per_block = per_block < 1 ? 1 : per_block > slots ? slots : per_block;
+  const int groups = (slots + per_block - 1) / per_block;
+  const int32_t *first = (a.B + kChunk - 1) / kChunk > kFuseChunks
+                             ? reinterpret_cast<const int32_t *>(a.chunk_col)
+                             : nullptr;
+  return launch_pdl(gather_kernel, dim3(a.B * groups), dim3(256), 0, s, x, a.ids, a.pos, first, a.meta,
+                    xp, zero_out, a.B, a.N, d, a.k, a.n_shared, per_block, pf);
 }
 
 cudaError_t launch_combine(const float *out, const int32_t *pos, const float *w,

@@ -32,8 +32,7 @@ constexpr int kStaticMaxTiles = kMaxN + kStaticMaxPairs / kTileTok + 1;
 constexpr size_t kOffTopTok = 0;
 constexpr size_t kOffCounts = kOffTopTok + up256(sizeof(int32_t) * kStaticMaxB * kMaxK);
 constexpr size_t kOffOffsets = kOffCounts + up256(sizeof(int32_t) * kMaxN);
-constexpr size_t kOffPerm = kOffOffsets + up256(sizeof(int32_t) * (kMaxN + 1));
-constexpr size_t kOffPos = kOffPerm + up256(sizeof(int32_t) * kStaticMaxPairs);
+constexpr size_t kOffPos = kOffOffsets + up256(sizeof(int32_t) * (kMaxN + 1));
 constexpr size_t kOffTiles = kOffPos + up256(sizeof(int32_t) * kStaticMaxPairs);
 constexpr size_t kOffMeta = kOffTiles + up256(sizeof(Tile) * kStaticMaxTiles);
 constexpr int kStaticChunks = (kStaticMaxB + kChunk - 1) / kChunk;
@@ -164,7 +163,6 @@ extern "C" int xshare_route_static(const float *scores, int B, int N, int k, int
   a.toptok = reinterpret_cast<int32_t *>(base + kOffTopTok);
   a.counts = reinterpret_cast<int32_t *>(base + kOffCounts);
   a.offsets = reinterpret_cast<int32_t *>(base + kOffOffsets);
-  a.perm = reinterpret_cast<int32_t *>(base + kOffPerm);
   a.pos = reinterpret_cast<int32_t *>(base + kOffPos);
   a.tiles = reinterpret_cast<Tile *>(base + kOffTiles);
   a.meta = reinterpret_cast<Meta *>(base + kOffMeta);

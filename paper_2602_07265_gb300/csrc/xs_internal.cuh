@@ -49,7 +49,6 @@ constexpr int kMaxB = 8192;     // tokens
 constexpr int kTileTok = 128;   // tokens of one expert handled by one FFN tile
 constexpr int kRouteThreads = 1024;
 constexpr int kChunk = 32;                   // tokens per selection CTA (= the column-sum chunk)
-constexpr int kScatterMaxN = 256;            // parallel stable scatter up to this many experts
 constexpr int kFuseChunks = 2;               // up to this many chunks the selection CTA also refines
 constexpr int kMaxShared = 8;                // shared experts
 constexpr int kGatherPrefetchBytes = 256 * 1024;  // L2 warm-up per gate/up CTA (packed weights)
@@ -108,7 +107,7 @@ struct Meta {
 
 // Byte offsets of every workspace region (256-byte aligned).
 struct Plan {
-  size_t h, p, mask, ids, w, toptok, counts, offsets, perm, pos, tiles, meta;
+  size_t h, p, mask, ids, w, toptok, counts, offsets, pos, tiles, meta;
   size_t chunk_col, chunk_marks, done, gs, rstat;
   size_t xp, act, out, ffn_part, ffn_cnt;
   size_t total;
@@ -133,16 +132,18 @@ struct RouteArgs {
   int32_t *toptok;       // [B, 16] per-token ranked top over E
   int32_t *counts;       // [N]
   int32_t *offsets;      // [N + 1]
-  int32_t *perm;         // [B * k]
-  int32_t *pos;          // [B * k] inverse of perm (row of pair t*k+s), -1 if unrouted
+  int32_t *pos;          // [B * k] row of pair t*k+s, -1 if unrouted (for more than
+                         // kFuseChunks chunks its rank in the chunk until the gather kernel)
   Tile *tiles;           // [max_tiles]
   Meta *meta;
   xs_stats *stats;       // nullable
   int32_t *counts_out;   // nullable caller copies
   int32_t *offsets_out;
   int32_t *perm_out;
-  float *chunk_col;      // [C][N] column-sum tree of each 32-token chunk
-  uint8_t *chunk_marks;  // [C][2][N] each chunk's warm-up / base marks and union marks
+  float *chunk_col;      // [C][N] column-sum tree of each 32-token chunk; after the
+                         // refinement the first row (int32) of every chunk and expert
+  uint8_t *chunk_marks;  // [C][2][N] each chunk's warm-up / base marks and union marks; in
+                         // the refinement the chunk's pairs per expert (first half)
   int32_t *done;         // [4] arrival counters (selection, refinement, union), zero at
                          // entry, and the selected-set flag (done[3])
   int32_t *zero_words;   // nullable: region cleared for the FFN kernels
@@ -179,9 +180,6 @@ cudaError_t launch_router_tc(const uint16_t *x, const float *Wg, float *h, int B
 cudaError_t launch_combine(const float *out, const int32_t *pos, const float *w,
                            const Meta *meta, const uint16_t *resid, uint16_t *y, int B, int d,
                            int k, int n_shared, cudaStream_t s);
-// Gathers the token rows of this call's FFN rows into xp; with expert
-// parallelism (zero_out != nullptr) it zeroes the rows of zero_out that
-// another rank computes.
 // What the gather kernel needs to warm L2 with the gate/up kernel's first
 // weights (packed weights only; pk == nullptr: no warm-up).
 struct GatherPf {
@@ -193,9 +191,11 @@ struct GatherPf {
   int grid;               // the gate/up kernel's grid
   int pf_bytes;           // bytes per gate/up CTA to prefetch
 };
-cudaError_t launch_gather(const uint16_t *x, const int32_t *perm, const Meta *meta,
-                          uint16_t *xp, float *zero_out, int max_rows, int B, int d, int k,
-                          const GatherPf &pf, cudaStream_t s);
+// Places the pairs of the routing `a` and gathers the token rows of this
+// call's FFN rows into xp; with expert parallelism (zero_out != nullptr) it
+// zeroes the rows of zero_out that another rank computes.
+cudaError_t launch_gather(const uint16_t *x, const RouteArgs &a, uint16_t *xp, float *zero_out, int d,
+                          int n_sms, const GatherPf &pf, cudaStream_t s);
 
 struct FfnArgs {
   const uint16_t *W_gate, *W_up, *W_down;
