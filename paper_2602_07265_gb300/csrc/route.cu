@@ -57,16 +57,40 @@ __device__ __forceinline__ float canonical_sum(const float *__restrict__ p, int 
 }
 
 // ---------------------------------------------------------------------------
-// Warp-wide ranking.  A warp ranks up to 32 Q candidates: lane l holds the
-// candidates l + 32 q (q < Q) as (key, index) pairs, sorted best first in
-// registers by a bitonic network; each round then takes the best head of all
-// lanes with two warp reductions (largest key, then smallest index among the
-// lanes holding it) and the winning lane pops its head.
+// Warp-wide ranking.  A warp ranks up to 32 Q candidates; lane l holds the
+// candidates l + 32 q (q < Q).  Each round takes the best head of all lanes
+// with two warp reductions (largest key, then smallest index among the lanes
+// holding it) and the winning lane moves on to its next one.
+//
+// Up to 8 candidates per lane the lane keeps (key, index) pairs sorted best
+// first in registers (a bitonic network).  At 32 that is 64 registers and 240
+// exchanges, which spilled (10 KB of spill stores in score_kernel<32>): the
+// lane then keeps the keys alone, unsorted, and the winner scans them for its
+// next best (one lane, about 100 instructions a round).  Routing at N = 1000,
+// B = 100 on GB300 (whole call): 136 -> 35.6 us.
+constexpr int kSortedQ = 8;
+
 template <int Q>
-struct LaneList {
+struct LaneList {   // Q <= kSortedQ
   uint32_t key[Q];
   int idx[Q];
 };
+template <>
+struct LaneList<32> {
+  uint32_t key[32];   // slot q: candidate j0 + lane + 32 q; 0 once taken
+  int j0;
+  uint32_t best;      // the lane's largest key and its (lowest) slot
+  int bq;
+};
+
+// Candidate index of slot q.
+template <int Q>
+__device__ __forceinline__ int lane_index(const LaneList<Q> &L, int q) {
+  if constexpr (Q <= kSortedQ)
+    return L.idx[q];
+  else
+    return L.j0 + static_cast<int>(threadIdx.x & 31) + 32 * q;
+}
 
 // Total order of every top-k and argmax: larger score first, equal scores ->
 // lower expert index.
@@ -74,26 +98,44 @@ __device__ __forceinline__ bool before(uint32_t ka, int ia, uint32_t kb, int ib)
   return ka > kb || (ka == kb && ia < ib);
 }
 
+// The lane's best slot of an unsorted list (the lowest of equal keys).
+template <int Q>
+__device__ __forceinline__ void lane_scan(LaneList<Q> &L) {
+  uint32_t m = L.key[0];
+#pragma unroll
+  for (int q = 1; q < Q; ++q) m = max(m, L.key[q]);
+  int b = 0;
+#pragma unroll
+  for (int q = Q - 1; q >= 0; --q) b = L.key[q] == m ? q : b;
+  L.best = m;
+  L.bq = b;
+}
+
+// Prepares a loaded list for lane_take.
 template <int Q>
 __device__ __forceinline__ void lane_sort(LaneList<Q> &L) {
+  if constexpr (Q > kSortedQ) {
+    lane_scan<Q>(L);
+  } else {
 #pragma unroll
-  for (int k = 2; k <= Q; k <<= 1) {
+    for (int k = 2; k <= Q; k <<= 1) {
 #pragma unroll
-    for (int j = k >> 1; j > 0; j >>= 1) {
+      for (int j = k >> 1; j > 0; j >>= 1) {
 #pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        const int l = i ^ j;
-        if (l > i) {
-          const bool first_best = (i & k) == 0;
-          const bool sw = first_best ? before(L.key[l], L.idx[l], L.key[i], L.idx[i])
-                                     : before(L.key[i], L.idx[i], L.key[l], L.idx[l]);
-          if (sw) {
-            const uint32_t tk = L.key[i];
-            L.key[i] = L.key[l];
-            L.key[l] = tk;
-            const int ti = L.idx[i];
-            L.idx[i] = L.idx[l];
-            L.idx[l] = ti;
+        for (int i = 0; i < Q; ++i) {
+          const int l = i ^ j;
+          if (l > i) {
+            const bool first_best = (i & k) == 0;
+            const bool sw = first_best ? before(L.key[l], L.idx[l], L.key[i], L.idx[i])
+                                       : before(L.key[i], L.idx[i], L.key[l], L.idx[l]);
+            if (sw) {
+              const uint32_t tk = L.key[i];
+              L.key[i] = L.key[l];
+              L.key[l] = tk;
+              const int ti = L.idx[i];
+              L.idx[i] = L.idx[l];
+              L.idx[l] = ti;
+            }
           }
         }
       }
@@ -107,18 +149,33 @@ template <int Q, class Emit>
 __device__ __forceinline__ int lane_take(LaneList<Q> &L, int count, Emit emit) {
   int r = 0;
   for (; r < count; ++r) {
-    const uint32_t mx = __reduce_max_sync(kFull, L.key[0]);
+    uint32_t head;
+    int head_idx;
+    if constexpr (Q <= kSortedQ) {
+      head = L.key[0];
+      head_idx = L.idx[0];
+    } else {
+      head = L.best;
+      head_idx = lane_index<Q>(L, L.bq);
+    }
+    const uint32_t mx = __reduce_max_sync(kFull, head);
     if (mx == 0u) break;
-    const uint32_t cand = (L.key[0] == mx) ? static_cast<uint32_t>(L.idx[0]) : 0xffffffffu;
+    const uint32_t cand = head == mx ? static_cast<uint32_t>(head_idx) : 0xffffffffu;
     const int win = static_cast<int>(__reduce_min_sync(kFull, cand));
     emit(r, win, key_score(mx));
-    if (L.key[0] == mx && L.idx[0] == win) {
+    if (head == mx && head_idx == win) {
+      if constexpr (Q <= kSortedQ) {
 #pragma unroll
-      for (int q = 0; q + 1 < Q; ++q) {
-        L.key[q] = L.key[q + 1];
-        L.idx[q] = L.idx[q + 1];
+        for (int q = 0; q + 1 < Q; ++q) {
+          L.key[q] = L.key[q + 1];
+          L.idx[q] = L.idx[q + 1];
+        }
+        L.key[Q - 1] = 0u;
+      } else {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) L.key[q] = q == L.bq ? 0u : L.key[q];
+        lane_scan<Q>(L);
       }
-      L.key[Q - 1] = 0u;
     }
   }
   return r;
@@ -146,7 +203,7 @@ __device__ __forceinline__ void lane_mark_top(const LaneList<Q> &L, int count, M
   if (count >= live) {
 #pragma unroll
     for (int q = 0; q < Q; ++q)
-      if (L.key[q] != 0u) mark(L.idx[q]);
+      if (L.key[q] != 0u) mark(lane_index<Q>(L, q));
     return;
   }
   uint32_t kmx = 0u, kmn = 0xffffffffu;
@@ -167,7 +224,7 @@ __device__ __forceinline__ void lane_mark_top(const LaneList<Q> &L, int count, M
   auto mark_from = [&](uint32_t c) {
 #pragma unroll
     for (int q = 0; q < Q; ++q)
-      if (L.key[q] >= c) mark(L.idx[q]);
+      if (L.key[q] >= c) mark(lane_index<Q>(L, q));
   };
   auto count_from = [&](uint32_t c) {
     int n = 0;
@@ -195,14 +252,14 @@ __device__ __forceinline__ void lane_mark_top(const LaneList<Q> &L, int count, M
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
     gt += L.key[q] > T ? 1 : 0;
-    if (L.key[q] > T) mark(L.idx[q]);
+    if (L.key[q] > T) mark(lane_index<Q>(L, q));
   }
   int need = count - static_cast<int>(__reduce_add_sync(kFull, static_cast<unsigned>(gt)));
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
     const bool tie = L.key[q] == T;
     const unsigned b = __ballot_sync(kFull, tie);
-    if (tie && __popc(b & ((1u << lane) - 1u)) < need) mark(L.idx[q]);
+    if (tie && __popc(b & ((1u << lane) - 1u)) < need) mark(lane_index<Q>(L, q));
     need -= __popc(b);
   }
 }
@@ -230,26 +287,31 @@ __device__ __forceinline__ float expert_tree(float (&v)[Q]) {
 template <int Q, class Val, class Live>
 __device__ __forceinline__ void lane_load(LaneList<Q> &L, int j0, int n, int lane, Val val,
                                           Live live) {
+  if constexpr (Q > kSortedQ) L.j0 = j0;
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
     const int j = j0 + lane + 32 * q;
-    L.idx[q] = j;
+    if constexpr (Q <= kSortedQ) L.idx[q] = j;
     L.key[q] = (lane + 32 * q < n && live(q, j)) ? score_key(val(q, j)) : 0u;
   }
 }
 
-// Moves each lane's best candidate to slot 0 (enough for a single take).
+// Prepares a loaded list for a single take: each lane's best candidate.
 template <int Q>
 __device__ __forceinline__ void lane_head(LaneList<Q> &L) {
+  if constexpr (Q > kSortedQ) {
+    lane_scan<Q>(L);
+  } else {
 #pragma unroll
-  for (int q = 1; q < Q; ++q) {
-    if (before(L.key[q], L.idx[q], L.key[0], L.idx[0])) {
-      const uint32_t tk = L.key[0];
-      L.key[0] = L.key[q];
-      L.key[q] = tk;
-      const int ti = L.idx[0];
-      L.idx[0] = L.idx[q];
-      L.idx[q] = ti;
+    for (int q = 1; q < Q; ++q) {
+      if (before(L.key[q], L.idx[q], L.key[0], L.idx[0])) {
+        const uint32_t tk = L.key[0];
+        L.key[0] = L.key[q];
+        L.key[q] = tk;
+        const int ti = L.idx[0];
+        L.idx[0] = L.idx[q];
+        L.idx[q] = ti;
+      }
     }
   }
 }
@@ -455,6 +517,9 @@ __device__ __forceinline__ void refine_tokens(const RouteArgs &a, const uint8_t 
   } else if (kQ > 4 && nq <= 4) {
     compact_selected(s_mask, a.N, s_list, s_wc);
     refine_tokens_q<(kQ > 4 ? 4 : kQ)>(a, s_list, nS, t_begin, t_end, kp, row, ids_s);
+  } else if (kQ > kSortedQ && nq <= kSortedQ) {
+    compact_selected(s_mask, a.N, s_list, s_wc);
+    refine_tokens_q<kSortedQ>(a, s_list, nS, t_begin, t_end, kp, row, ids_s);
   } else {
     refine_tokens_masked<kQ>(a, s_mask, t_begin, t_end, kp, row, ids_s);
   }
