@@ -83,6 +83,7 @@ RouteArgs route_args(const Plan &pl, void *ws, int B, int N, int k, int budget, 
   a.m_g = prm->m_g > N ? N : prm->m_g;
   a.tau = prm->tau;
   a.sparse = (mode != XS_MODE_TOPK) ? prm->sparse_scores : 0;
+  a.tile_tok = kTileTok;
   a.gs = at<float>(ws, pl.gs);
   a.p = at<float>(ws, pl.p);
   a.mask = at<uint8_t>(ws, pl.mask);
@@ -255,6 +256,10 @@ int xs::forward_impl(const FwdCall &c, FwdStep step) {
   a.zero_words = at<int32_t>(workspace, pl.ffn_cnt);
   a.zero_count = (int)ffn_cnt_words(pl.max_tiles, B, d, F);
   a.n_shared = n_shared;
+  // At most this many experts can be selected (BATCH: warm-up and budget).
+  const long long sel_max = c.mode == XS_MODE_BATCH ? static_cast<long long>(B) * c.prm->k0 + c.budget : N;
+  const bool ffn_pairs = ffn_use_pairs(static_cast<long long>(B) * k, static_cast<int>(sel_max < N ? sel_max : N));
+  if (ffn_pairs) a.tile_tok = kPairTok;
 
   FfnArgs f;
   std::memset(&f, 0, sizeof(f));
@@ -286,6 +291,7 @@ int xs::forward_impl(const FwdCall &c, FwdStep step) {
   f.max_rows = pl.max_rows;
   f.max_tiles = pl.max_tiles;
   f.n_sms = sms;
+  f.n_weights = ep ? N / c.ep_ranks : N;
   f.expert_base = ep ? c.ep_rank * (N / c.ep_ranks) : 0;
 
   auto mark = [&](int i) {
@@ -316,7 +322,7 @@ int xs::forward_impl(const FwdCall &c, FwdStep step) {
   // the selected set is known (packed weights, without expert parallelism).
   GatherPf pf;
   std::memset(&pf, 0, sizeof(pf));
-  if (packed && !ep) {
+  if (packed && !ep && !ffn_pairs) {
     pf.ready = a.done + 3;
     pf.mask = a.mask;
     pf.pk = static_cast<const uint8_t *>(c.P_gate_up);
@@ -333,8 +339,10 @@ int xs::forward_impl(const FwdCall &c, FwdStep step) {
           cudaSuccess ||
       !mark(4))
     return XS_ERR_CUDA;
-  if (launch_ffn_gate_up(f, s) != cudaSuccess || !mark(5)) return XS_ERR_CUDA;
-  if (launch_ffn_down(f, s) != cudaSuccess || !mark(6)) return XS_ERR_CUDA;
+  if ((ffn_pairs ? launch_ffn_pair_gate_up(f, s) : launch_ffn_gate_up(f, s)) != cudaSuccess || !mark(5))
+    return XS_ERR_CUDA;
+  if ((ffn_pairs ? launch_ffn_pair_down(f, s) : launch_ffn_down(f, s)) != cudaSuccess || !mark(6))
+    return XS_ERR_CUDA;
   if (ep) {
     if (c.topk_w != nullptr &&
         cudaMemcpyAsync(c.topk_w, a.w, static_cast<size_t>(B) * k * sizeof(float),

@@ -525,18 +525,24 @@ __device__ __forceinline__ void refine_tokens(const RouteArgs &a, const uint8_t 
   }
 }
 
-// FFN tiles of expert e's run of cnt rows from row0, as tiles[tile0 ...].
-// tile_count() says how many.
-__device__ __forceinline__ int tile_count(int cnt) { return (cnt + kTileTok - 1) / kTileTok; }
+// FFN tiles of a run of cnt rows: full ones and a rest for ffn_tc.cu
+// (kTileTok tokens); for ffn_pair.cu, whose tiles stream the expert's weights
+// once each, even shares in steps of the MMA's 32 tokens.
+__device__ __forceinline__ int tile_count(int cnt, int tile_tok) { return (cnt + tile_tok - 1) / tile_tok; }
 
-__device__ __forceinline__ void write_tiles(Tile *tiles, int tile0, int e, int row0, int cnt) {
-  for (int tt = 0; tt * kTileTok < cnt; ++tt) {
+// Writes the tiles of expert e's rows [row0, row0 + cnt) as tiles[tile0 ...].
+__device__ __forceinline__ void write_tiles(Tile *tiles, int tile0, int e, int row0, int cnt, int tile_tok) {
+  const int n = tile_count(cnt, tile_tok), steps = (cnt + 31) / 32;
+  for (int i = 0; i < n; ++i) {
+    const bool even = tile_tok != kTileTok;
+    const int lo = even ? steps * i / n * 32 : i * tile_tok;
+    const int hi = min(cnt, even ? steps * (i + 1) / n * 32 : lo + tile_tok);
     Tile tl;
     tl.expert = e;
-    tl.row0 = row0 + tt * kTileTok;
-    tl.ntok = min(kTileTok, cnt - tt * kTileTok);
+    tl.row0 = row0 + lo;
+    tl.ntok = hi - lo;
     tl.pad = 0;
-    tiles[tile0 + tt] = tl;
+    tiles[tile0 + i] = tl;
   }
 }
 
@@ -606,7 +612,7 @@ __device__ void build_offsets(const RouteArgs &a, int32_t *s_part, int32_t *s_of
       s_part[q * Np + tid] = n_e;
       n_e += x;
     }
-  int v[3] = {n_e, tile_count(n_e), n_e > 0 ? 1 : 0}, tot[3];
+  int v[3] = {n_e, tile_count(n_e, a.tile_tok), n_e > 0 ? 1 : 0}, tot[3];
   block_scan3(v, tot, s_tmp);
   if (tid < N) {
     s_off[tid] = v[0];
@@ -614,7 +620,7 @@ __device__ void build_offsets(const RouteArgs &a, int32_t *s_part, int32_t *s_of
     a.offsets[tid] = v[0];
     if (a.counts_out) a.counts_out[tid] = n_e;
     if (a.offsets_out) a.offsets_out[tid] = v[0];
-    write_tiles(a.tiles, v[1], tid, v[0], n_e);
+    write_tiles(a.tiles, v[1], tid, v[0], n_e, a.tile_tok);
   }
   // This call's FFN work (Sec. 5): the tiles and rows of the experts of
   // group ep_rank, a contiguous index range, hence contiguous tiles and
@@ -638,7 +644,7 @@ __device__ void build_offsets(const RouteArgs &a, int32_t *s_part, int32_t *s_of
         m->ffn_t1 = tot[1];
         m->row1 = tot[0];
       }
-      const int own_shared = g == 0 ? 1 : 0, shared_tiles = a.n_shared * tile_count(B);
+      const int own_shared = g == 0 ? 1 : 0, shared_tiles = a.n_shared * tile_count(B, a.tile_tok);
       m->ffn_s0 = tot[1];
       m->ffn_s1 = tot[1] + own_shared * shared_tiles;
       m->srows = own_shared;
@@ -660,7 +666,7 @@ __device__ void build_offsets(const RouteArgs &a, int32_t *s_part, int32_t *s_of
   }
   // Shared experts: every token, in token order, after the routed pairs.
   for (int j = tid; j < a.n_shared; j += blockDim.x)
-    write_tiles(a.tiles, tot[1] + j * tile_count(B), N + j, tot[0] + j * B, B);
+    write_tiles(a.tiles, tot[1] + j * tile_count(B, a.tile_tok), N + j, tot[0] + j * B, B, a.tile_tok);
   __syncthreads();
   if (e < N && part < parts) {
     int run = s_off[e] + s_part[part * Np + e];

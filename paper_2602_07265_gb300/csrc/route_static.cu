@@ -173,6 +173,7 @@ extern "C" int xshare_route_static(const float *scores, int B, int N, int k, int
   a.chunk_col = reinterpret_cast<float *>(base + kOffChunkCol);
   a.chunk_marks = reinterpret_cast<uint8_t *>(base + kOffChunkMarks);
   a.done = reinterpret_cast<int32_t *>(base + kOffDone);
+  a.tile_tok = kTileTok;
   a.zero_words = nullptr;
   a.zero_count = 0;
   // The three arrival counters must start at zero; every other scratch word is

@@ -14,4 +14,10 @@ bool encode_tmap_2d(CUtensorMap *m, CUtensorMapDataType dtype, uint32_t elem_byt
                     const void *base, uint64_t inner, uint64_t outer, uint32_t box_inner,
                     uint32_t box_outer, CUtensorMapSwizzle swizzle);
 
+// A tensor of `rank` <= 5 dimensions (innermost first), byte strides of
+// dimensions 1 .. rank - 1.
+bool encode_tmap(CUtensorMap *m, CUtensorMapDataType dtype, const void *base, int rank,
+                 const uint64_t *dims, const uint64_t *strides, const uint32_t *box,
+                 CUtensorMapSwizzle swizzle);
+
 }  // namespace xs

@@ -46,7 +46,8 @@ cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, size_t 
 constexpr int kMaxN = 1024;     // experts
 constexpr int kMaxK = 16;       // top-k and warm-up k0
 constexpr int kMaxB = 8192;     // tokens
-constexpr int kTileTok = 128;   // tokens of one expert handled by one FFN tile
+constexpr int kTileTok = 128;   // tokens of one expert handled by one tile of ffn_tc.cu
+constexpr int kPairTok = 256;   // and of ffn_pair.cu
 constexpr int kRouteThreads = 1024;
 constexpr int kChunk = 32;                   // tokens per selection CTA (= the column-sum chunk)
 constexpr int kFuseChunks = 2;               // up to this many chunks the selection CTA also refines
@@ -74,7 +75,16 @@ __host__ __device__ inline int ffn_ctas(long long U, int KI, int grid) {
   return static_cast<int>(want < grid ? want : grid);
 }
 
-// One FFN work tile: up to kTileTok consecutive rows of the permuted pair
+// Batches with at least this many routed pairs per expert that can be
+// selected take the CTA-pair FFN kernels (ffn_pair.cu).
+// Both sides on GB300, plain top-k, whole layer, ffn_tc.cu | ffn_pair.cu at 48,
+// 64, 96 and 128 pairs an expert: N = 64, d = 2048, F = 1024: 168 | 173, 179 |
+// 179, 207 | 191, 286 | 205 us; N = 128, F = 768: 248 | 257, 264 | 265 us at 48
+// and 64, 416 | 319 us at 128.  Below, the weights' stream is the bound and
+// ffn_tc.cu splits it over the SMs without a remainder.
+constexpr int kPairMinTok = 64;
+
+// One FFN work tile: up to kTileTok (kPairTok) consecutive rows of the permuted pair
 // list, all routed to `expert`.  Experts N .. N + n_shared - 1 are the shared
 // experts; their rows follow the routed pairs: row n_pairs + j * B + t is
 // token t's pass through shared expert j.
@@ -151,6 +161,7 @@ struct RouteArgs {
   void *const *events;   // nullable: events[0] is recorded between the two kernels
   int fuse_refine;       // set by launch_route: refinement runs in the selection kernel
   int n_shared;          // shared-expert tiles appended after the routed ones
+  int tile_tok;          // tokens per FFN tile: kTileTok or kPairTok
   const int32_t *router_status;  // nullable: per-CTA status of the tensor-core router
   int router_ctas;
   int ep_ranks, ep_rank;  // expert parallelism: the FFN work of group ep_rank of ep_ranks (0: all)
@@ -212,11 +223,17 @@ struct FfnArgs {
   void *part;            // partial-sum scratch
   int32_t *cnt;          // arrival counters (cleared by the routing kernel)
   int N, d, F, max_rows, max_tiles, n_sms;
+  int n_weights;         // routed experts that the weights hold (N, or the rank's share)
   int expert_base;       // routed expert e uses weights e - expert_base (expert parallelism)
 };
 
 cudaError_t launch_ffn_gate_up(const FfnArgs &a, cudaStream_t s);
 cudaError_t launch_ffn_down(const FfnArgs &a, cudaStream_t s);
+// The same on CTA pairs, for tiles of up to kPairTok tokens; whether a batch of
+// `pairs` routed pairs over at most `experts` experts takes them.
+bool ffn_use_pairs(long long pairs, int experts);
+cudaError_t launch_ffn_pair_gate_up(const FfnArgs &a, cudaStream_t s);
+cudaError_t launch_ffn_pair_down(const FfnArgs &a, cudaStream_t s);
 size_t ffn_part_bytes(int n_sms);
 // Packs W0 (and W1) [n][M][K] bf16 into 128 x 64 swizzled tiles (pack.cu).
 cudaError_t launch_pack(const uint16_t *W0, const uint16_t *W1, void *P, int n, int M, int K,

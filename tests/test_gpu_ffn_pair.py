@@ -1,0 +1,47 @@
+"""The CTA-pair FFN kernels (many tokens per expert) against the oracle, on
+plain and packed weights (the same bits), at the edges of their tiles: token
+counts around 32 and 256, an odd number of 128-row blocks in d, one K step
+pair, experts with few tokens beside full ones, shared experts, and a rank of
+an expert-parallel layer."""
+import pytest
+import torch
+
+from paper_2602_07265_gb300 import workloads as W
+from test_gpu_ep import run_ep, run_one_gpu
+from test_gpu_forward import compare, gpu_forward
+from test_gpu_route import X  # noqa: F401  (fixture)
+
+pytestmark = pytest.mark.gpu
+
+
+def _inputs(w, n_shared):
+    x, W_g = W.router_inputs(w, seed=5)
+    weights = W.expert_weights(w, seed=5, device="cuda")
+    return x, W_g, weights, W.shared_expert_weights(w, n_shared, seed=5) if n_shared else None
+
+
+# With N == k every expert gets exactly B tokens; otherwise the counts spread.
+@pytest.mark.parametrize("N,k,d,F,B,mode,n_shared", [
+    (2, 2, 128, 128, 64, W.MODE_TOPK, 0), (4, 4, 384, 256, 255, W.MODE_TOPK, 0),
+    (2, 2, 256, 384, 256, W.MODE_TOPK, 1), (3, 3, 640, 128, 257, W.MODE_TOPK, 0),
+    (8, 2, 256, 256, 1000, W.MODE_TOPK, 2), (32, 4, 128, 384, 700, W.MODE_BATCH, 0),
+    (16, 3, 2048, 256, 513, W.MODE_HIER, 0)])
+def test_pair_forward(X, N, k, d, F, B, mode, n_shared):  # noqa: F811
+    w = W.TINY.with_(N=N, k=k, d=d, F=F, B=B, mode=mode, budget=6, k0=0, m_r=2,
+                     tokens_per_request=3 if mode == W.MODE_HIER else 1, x_kind="domains")
+    x, W_g, weights, shared = _inputs(w, n_shared)
+    g = gpu_forward(X, w, x, W_g, weights, shared=shared)
+    assert g["stats"]["status"] == 0
+    compare(w, g, x, W_g, weights, shared=shared)
+    pk, ps = X.Packed(*weights), X.Packed(*shared) if shared else None
+    y = run_one_gpu(X, w, x, W_g, pk, shared=ps)["y"]
+    assert torch.equal(y.cpu().double(), torch.from_numpy(g["y"])), "packed and plain weights differ"
+
+
+def test_pair_expert_parallel(X):  # noqa: F811
+    w = W.TINY.with_(N=8, k=2, d=256, F=256, B=900, mode=W.MODE_TOPK, x_kind="domains")
+    x, W_g, weights, shared = _inputs(w, 1)
+    pk, ps = X.Packed(*weights), X.Packed(*shared)
+    one = run_one_gpu(X, w, x, W_g, pk, shared=ps)["y"]
+    y = run_ep(X, w, x, W_g, pk, 4, shared=ps)[0]
+    assert torch.equal(y, one)   # no unit is cut: every row is the same bits on any rank
