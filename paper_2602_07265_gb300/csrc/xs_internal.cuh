@@ -201,6 +201,7 @@ struct GatherPf {
   int stage_bytes;        // packed bytes per step (gate and up tiles)
   int grid;               // the gate/up kernel's grid
   int pf_bytes;           // bytes per gate/up CTA to prefetch
+  int max_used;           // at most this many experts get a token (the batch's pairs)
 };
 // Places the pairs of the routing `a` and gathers the token rows of this
 // call's FFN rows into xp; with expert parallelism (zero_out != nullptr) it
