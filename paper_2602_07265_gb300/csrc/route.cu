@@ -916,7 +916,7 @@ __global__ void __launch_bounds__(kRouteThreads, 1) score_kernel(RouteArgs a) {
   __shared__ uint8_t s_union[kMaxN];    // union CTAs: plain top-k union marks
   __shared__ float s_col[kMaxN];
   __shared__ int32_t s_gl[kMaxN + 1];
-  __shared__ int32_t s_top[kChunk][kMaxK];
+  __shared__ int32_t s_top[2 * kChunk - 1][kMaxK];
   __shared__ int32_t s_scal[4];
   __shared__ uint32_t s_counts[kMaxN];  // token masks of the permutation, when it runs in
   __shared__ uint32_t s_cursor[kMaxN];  // this kernel: tokens 32-63, tokens 0-31
@@ -940,9 +940,15 @@ __global__ void __launch_bounds__(kRouteThreads, 1) score_kernel(RouteArgs a) {
   // top-k for Sec. 2.2's gating values when the column scores are sparse.
   const int kk = a.sparse ? max(k, a.k0) : a.k0;
   const bool hier = a.mode == XS_MODE_HIER;
-  // HIER requests that lie inside one chunk are selected here (Algorithm 3);
-  // otherwise the selection step does it from the full score matrix.
-  const bool hier_here = hier && a.T <= kChunk && kChunk % a.T == 0;
+  // HIER requests are selected by the CTA whose chunk they begin in
+  // (Algorithm 3): it also takes the scores of their tokens past the chunk
+  // (rows kChunk .. hier_rows - 1 of ps).  Without that (hier_rows == 0:
+  // longer requests, or more rows than shared memory holds) the selection
+  // step does it from the full score matrix, alone (layer forward at N = 128,
+  // d = 2048, F = 768, T = 5, that way and this way: B = 125 178.7 and 175.4
+  // us, B = 600 276 and 245.5 us).
+  const bool hier_here = hier && a.hier_rows > 0;
+  const int rows = hier_here ? a.hier_rows : kChunk;
 
   for (int j = tid; j < N; j += blockDim.x) s_base[j] = 0;
   if (a.zero_words != nullptr)
@@ -950,15 +956,16 @@ __global__ void __launch_bounds__(kRouteThreads, 1) score_kernel(RouteArgs a) {
   __syncthreads();
 
   // ---- per token: scores (a2) and ranking over E (a3) ----
-  for (int w = warp; w < kChunk; w += nwarps) {
+  for (int w = warp; w < rows; w += nwarps) {
     float *prow_s = ps + w * N;
-    if (w >= nt) {  // zero rows pad the last chunk's tree
-      for (int j = lane; j < N; j += 32) prow_s[j] = 0.f;
+    const int t = t0 + w;
+    const bool own = w < kChunk;  // else a token of the next chunk's, for a request begun here
+    if (t >= B) {  // zero rows pad the last chunk's tree
+      for (int j = lane; own && j < N; j += 32) prow_s[j] = 0.f;
       continue;
     }
-    const int t = t0 + w;
     float vals[kQ];
-    token_scores<kQ>(a, t, lane, vals, true);
+    token_scores<kQ>(a, t, lane, vals, own);
 #pragma unroll
     for (int q = 0; q < kQ; ++q)
       if (lane + 32 * q < N) prow_s[lane + 32 * q] = vals[q];
@@ -977,10 +984,10 @@ __global__ void __launch_bounds__(kRouteThreads, 1) score_kernel(RouteArgs a) {
       if (lane == 0) {
         if (r < a.k0) {
           s_top[w][r] = id;
-          if (hier)
-            top[r] = id;
-          else
+          if (!hier)
             s_base[id] = 1;
+          else if (own)
+            top[r] = id;
         }
       }
       if (r < k) {
@@ -1030,11 +1037,11 @@ __global__ void __launch_bounds__(kRouteThreads, 1) score_kernel(RouteArgs a) {
       a.chunk_col[(size_t)c * N + j] = v[0];
   }
 
-  // ---- HIER: Algorithm 3 for the requests inside this chunk ----
+  // ---- HIER: Algorithm 3 for the requests that begin in this chunk ----
   if (hier_here) {
     const int T = a.T;
-    for (int r = warp; r * T < nt; r += nwarps) {
-      const int r0 = r * T, r1 = min(r0 + T, nt);
+    for (int r = (t0 + T - 1) / T + warp; r * T < t0 + nt; r += nwarps) {
+      const int r0 = r * T - t0, r1 = r0 + T;
       float sc[kQ];
       uint32_t excl = 0;
 #pragma unroll
@@ -1088,7 +1095,7 @@ __global__ void __launch_bounds__(kRouteThreads, 1) score_kernel(RouteArgs a) {
   if (!one_pass) __syncthreads();
 
   if (hier && !hier_here) {
-    // Requests cross chunk boundaries: Algorithm 3 from the full score matrix.
+    // Algorithm 3 from the full score matrix.
     const int T = a.T, R = B / T;
     for (int r = warp; r < R; r += nwarps) {
       const int r0 = r * T, r1 = r0 + T;
@@ -1641,7 +1648,10 @@ cudaError_t launch_route_q(const RouteArgs &a, cudaStream_t s) {
   const int C = (a.B + kChunk - 1) / kChunk;
   RouteArgs b = a;
   b.fuse_refine = C <= kFuseChunks ? 1 : 0;
-  const int dyn1 = kChunk * a.N * 4;
+  // HIER: rows for the tokens that a request begun in a chunk has past it.
+  const int need = a.mode != XS_MODE_HIER || a.T > kChunk ? 0 : kChunk % a.T == 0 ? kChunk : kChunk + a.T - 1;
+  b.hier_rows = need * a.N * 4 <= kScoreRowBytes ? need : 0;
+  const int dyn1 = (b.hier_rows > kChunk ? b.hier_rows : kChunk) * a.N * 4;
   cudaError_t e = cudaFuncSetAttribute(score_kernel<kQ>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, dyn1);
   if (e != cudaSuccess) return e;

@@ -50,6 +50,7 @@ constexpr int kTileTok = 128;   // tokens of one expert handled by one tile of f
 constexpr int kPairTok = 256;   // and of ffn_pair.cu
 constexpr int kRouteThreads = 1024;
 constexpr int kChunk = 32;                   // tokens per selection CTA (= the column-sum chunk)
+constexpr int kScoreRowBytes = 190 * 1024;   // score rows of a selection CTA at most
 constexpr int kFuseChunks = 2;               // up to this many chunks the selection CTA also refines
 constexpr int kMaxShared = 8;                // shared experts
 constexpr int kGatherPrefetchBytes = 256 * 1024;  // L2 warm-up per gate/up CTA (packed weights)
@@ -160,6 +161,7 @@ struct RouteArgs {
   int zero_count;
   void *const *events;   // nullable: events[0] is recorded between the two kernels
   int fuse_refine;       // set by launch_route: refinement runs in the selection kernel
+  int hier_rows;         // set by launch_route: score rows per selection CTA for HIER, or 0
   int n_shared;          // shared-expert tiles appended after the routed ones
   int tile_tok;          // tokens per FFN tile: kTileTok or kPairTok
   const int32_t *router_status;  // nullable: per-CTA status of the tensor-core router
