@@ -428,6 +428,32 @@ __device__ __forceinline__ int compact_selected(const uint8_t *s_mask, int N, in
 
 static_assert(kRouteThreads >= kMaxN, "compact_selected takes one thread per expert");
 
+// Token t's best kp candidates of a loaded list into its slots, with the
+// renormalised weights (a6); one warp.  ids_row: nullable copy of the ids.
+template <int Q>
+__device__ __forceinline__ void take_slots(const RouteArgs &a, LaneList<Q> &L, int t, int kp, int32_t *ids_row) {
+  const int lane = threadIdx.x & 31, k = a.k;
+  lane_sort<Q>(L);
+  int my_id = -1;  // lane s keeps slot s
+  float my_v = 0.f;
+  float D = 0.f;
+  const int got = lane_take<Q>(L, kp, [&](int r, int id, float v) {
+    if (lane == r) {
+      my_id = id;
+      my_v = v;
+    }
+    D = __fadd_rn(D, v);  // slot order, identical on every lane
+  });
+  if (lane < k) {
+    float wv = 0.f;
+    if (lane < got) wv = (D > 0.f) ? __fdiv_rn(my_v, D) : __fdiv_rn(1.f, (float)got);
+    const int id = lane < got ? my_id : -1;
+    a.ids[(size_t)t * k + lane] = id;
+    if (ids_row) ids_row[lane] = id;
+    a.w[(size_t)t * k + lane] = wv;
+  }
+}
+
 // Per token t in [t_begin, t_end), one warp each: Top k'(G_t, S) with the
 // renormalised weights (a6); row(t) points at the token's scores.  Lane l
 // ranks the experts s_list[l + 32 q] of S (q < Q, Q * 32 >= |S|).
@@ -436,7 +462,6 @@ __device__ __forceinline__ void refine_tokens_q(const RouteArgs &a, const int32_
                                                 int t_begin, int t_end, int kp, Row row,
                                                 int32_t *ids_s) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  const int k = a.k;
   for (int t = t_begin + warp; t < t_end; t += nwarps) {
     const float *prow = row(t);
     LaneList<Q> L;
@@ -447,24 +472,7 @@ __device__ __forceinline__ void refine_tokens_q(const RouteArgs &a, const int32_
       L.idx[q] = e;
       L.key[q] = i < nS ? score_key(prow[e]) : 0u;
     }
-    lane_sort<Q>(L);
-    int my_id = -1;  // lane s keeps slot s
-    float my_v = 0.f;
-    float D = 0.f;
-    const int got = lane_take<Q>(L, kp, [&](int r, int id, float v) {
-      if (lane == r) {
-        my_id = id;
-        my_v = v;
-      }
-      D = __fadd_rn(D, v);  // slot order, identical on every lane
-    });
-    if (lane < k) {
-      float wv = 0.f;
-      if (lane < got) wv = (D > 0.f) ? __fdiv_rn(my_v, D) : __fdiv_rn(1.f, (float)got);
-      a.ids[(size_t)t * k + lane] = (lane < got) ? my_id : -1;
-      if (ids_s) ids_s[(t - t_begin) * k + lane] = (lane < got) ? my_id : -1;
-      a.w[(size_t)t * k + lane] = wv;
-    }
+    take_slots<Q>(a, L, t, kp, ids_s ? ids_s + (t - t_begin) * a.k : nullptr);
   }
 }
 
@@ -474,30 +482,13 @@ __device__ __forceinline__ void refine_tokens_masked(const RouteArgs &a, const u
                                                      int t_begin, int t_end, int kp, Row row,
                                                      int32_t *ids_s) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  const int N = a.N, k = a.k;
+  const int N = a.N;
   for (int t = t_begin + warp; t < t_end; t += nwarps) {
     const float *prow = row(t);
     LaneList<kQ> L;
     lane_load<kQ>(L, 0, N, lane, [&](int, int j) { return prow[j]; },
                   [&](int, int j) { return s_mask[j] != 0; });
-    lane_sort<kQ>(L);
-    int my_id = -1;
-    float my_v = 0.f;
-    float D = 0.f;
-    const int got = lane_take<kQ>(L, kp, [&](int r, int id, float v) {
-      if (lane == r) {
-        my_id = id;
-        my_v = v;
-      }
-      D = __fadd_rn(D, v);
-    });
-    if (lane < k) {
-      float wv = 0.f;
-      if (lane < got) wv = (D > 0.f) ? __fdiv_rn(my_v, D) : __fdiv_rn(1.f, (float)got);
-      a.ids[(size_t)t * k + lane] = (lane < got) ? my_id : -1;
-      if (ids_s) ids_s[(t - t_begin) * k + lane] = (lane < got) ? my_id : -1;
-      a.w[(size_t)t * k + lane] = wv;
-    }
+    take_slots<kQ>(a, L, t, kp, ids_s ? ids_s + (t - t_begin) * a.k : nullptr);
   }
 }
 
@@ -1312,6 +1303,69 @@ __global__ void __launch_bounds__(kRouteThreads, 1) refine_kernel(RouteArgs a) {
   build_offsets(a, reinterpret_cast<int32_t *>(s_tm), s_chunk, s_tmp);
 }
 
+// TOPK (S = E) for more than kFuseChunks chunks in one kernel: nothing has to
+// be known of the other tokens, so the CTA of a chunk takes the scores and the
+// slots of its tokens at once, and the plain top-k union is the used experts.
+// Layer forward on GB300, score_kernel and refine_kernel -> this: N = 64, d =
+// 2048, F = 1024: B = 128 153.2 -> 146.9, B = 2048 274.1 -> 265.5 us; N = 128,
+// F = 768: B = 256 219.0 -> 210.9, B = 2048 308.4 -> 298.0 us.
+template <int kQ>
+__global__ void __launch_bounds__(kRouteThreads, 1) topk_kernel(RouteArgs a) {
+  __shared__ uint32_t s_tm[kMaxN];      // token masks of the chunk, then build_offsets scratch
+  __shared__ int32_t s_chunk[kMaxN];
+  __shared__ int32_t s_ids[kChunk * kMaxK];
+  __shared__ int32_t s_tmp[200];
+  __shared__ int32_t s_last;
+  __shared__ int s_rflag;               // a router CTA reported a timeout
+
+  pdl_wait();
+  pdl_trigger();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
+  const int B = a.B, N = a.N, k = a.k;
+  const int C = chunk_count(B), c = blockIdx.x;
+  const int t0 = c * kChunk, nt = min(kChunk, B - t0);
+  if (tid == 0) s_rflag = 0;
+  if (c == 0 && warp == 0) {  // the selected set, then its flag (see score_kernel)
+    for (int j = lane; j < N; j += 32) a.mask[j] = 1;
+    __syncwarp();
+    if (lane == 0) *reinterpret_cast<volatile int32_t *>(a.done + 3) = 1;
+  }
+  for (int j = tid; j < N; j += blockDim.x) s_tm[j] = 0u;
+  if (a.zero_words != nullptr)
+    for (int i = c * blockDim.x + tid; i < a.zero_count; i += C * blockDim.x) a.zero_words[i] = 0;
+  for (int w = warp; w < nt; w += nwarps) {
+    float vals[kQ];
+    token_scores<kQ>(a, t0 + w, lane, vals, true);
+    LaneList<kQ> L;
+    lane_load<kQ>(L, 0, N, lane, [&](int q, int) { return vals[q]; }, [](int, int) { return true; });
+    take_slots<kQ>(a, L, t0 + w, k, s_ids + w * k);
+  }
+  __syncthreads();
+  publish_chunk(a, s_ids, s_tm, c, nt);
+
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) s_last = (atomicAdd(&a.done[1], 1) == C - 1) ? 1 : 0;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  for (int i = tid; i < a.router_ctas; i += blockDim.x)
+    if (__ldcg(a.router_status + i) != 0) s_rflag = 1;
+  __syncthreads();
+  if (tid == 0) {
+    Meta *m = a.meta;
+    m->kprime = k;
+    m->n_selected = N;
+    m->max_group_load = N / a.G;
+    m->status = s_rflag ? XS_DEV_TIMEOUT : XS_DEV_OK;
+  }
+  build_offsets(a, reinterpret_cast<int32_t *>(s_tm), s_chunk, s_tmp);
+  if (tid == 0) {
+    a.meta->union_topk = a.meta->n_used;
+    if (a.stats) a.stats->union_topk = a.meta->n_used;
+  }
+}
+
 // Row of pair q = t * k + s: final in pos[q] for up to kFuseChunks chunks
 // (first == nullptr), else its rank plus the first row of (chunk, expert).
 __device__ __forceinline__ int pair_row(const int32_t *ids, const int32_t *pos, const int32_t *first,
@@ -1643,17 +1697,30 @@ __global__ void __launch_bounds__(256) combine_kernel(const float *__restrict__ 
 
 }  // namespace
 
+static cudaError_t launch_scatter(const RouteArgs &a, cudaStream_t s) {
+  const int P = a.B * a.k;
+  return launch_pdl(scatter_kernel, dim3((P + 255) / 256), dim3(256), 0, s, a.ids, a.pos,
+                    reinterpret_cast<const int32_t *>(a.chunk_col), a.perm_out, P, a.N, a.k);
+}
+
 template <int kQ>
 cudaError_t launch_route_q(const RouteArgs &a, cudaStream_t s) {
   const int C = (a.B + kChunk - 1) / kChunk;
   RouteArgs b = a;
   b.fuse_refine = C <= kFuseChunks ? 1 : 0;
+  cudaError_t e;
+  if (a.mode == XS_MODE_TOPK && !b.fuse_refine) {
+    e = launch_pdl(topk_kernel<kQ>, dim3(C), dim3(kRouteThreads), 0, s, b);
+    if (e == cudaSuccess && a.events != nullptr)
+      e = cudaEventRecord(reinterpret_cast<cudaEvent_t>(a.events[0]), s);
+    if (e != cudaSuccess || a.perm_out == nullptr) return e;
+    return launch_scatter(a, s);
+  }
   // HIER: rows for the tokens that a request begun in a chunk has past it.
   const int need = a.mode != XS_MODE_HIER || a.T > kChunk ? 0 : kChunk % a.T == 0 ? kChunk : kChunk + a.T - 1;
   b.hier_rows = need * a.N * 4 <= kScoreRowBytes ? need : 0;
   const int dyn1 = (b.hier_rows > kChunk ? b.hier_rows : kChunk) * a.N * 4;
-  cudaError_t e = cudaFuncSetAttribute(score_kernel<kQ>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, dyn1);
+  e = cudaFuncSetAttribute(score_kernel<kQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn1);
   if (e != cudaSuccess) return e;
   e = launch_pdl(score_kernel<kQ>, dim3(2 * C), dim3(kRouteThreads), (size_t)dyn1, s, b);
   if (e != cudaSuccess) return e;
@@ -1667,9 +1734,7 @@ cudaError_t launch_route_q(const RouteArgs &a, cudaStream_t s) {
   }
   e = launch_pdl(refine_kernel<kQ>, dim3(C), dim3(kRouteThreads), 0, s, b);
   if (e != cudaSuccess || a.perm_out == nullptr) return e;
-  const int P = a.B * a.k;
-  return launch_pdl(scatter_kernel, dim3((P + 255) / 256), dim3(256), 0, s, a.ids, a.pos,
-                    reinterpret_cast<const int32_t *>(a.chunk_col), a.perm_out, P, a.N, a.k);
+  return launch_scatter(a, s);
 }
 
 cudaError_t launch_route(const RouteArgs &a, cudaStream_t s) {
