@@ -27,9 +27,13 @@
 // round-to-nearest addition per stage, while the next stages are
 // multiplied into up to seven other TMEM buffers.
 //
-// Roles (320 threads): warp 0 lane 0 issues TMA, warp 1 lane 0 issues the
-// MMAs, warps 2-5 convert the weight planes, warps 6-9 drain the TMEM
-// buffers.  Every mbarrier wait is bounded; every thread reaches both
+// Roles (448 threads): warp 0 lane 0 issues TMA, warp 1 lane 0 issues the
+// MMAs, warps 2-5 and 6-9 convert the weight planes of the even and the odd
+// K steps (the conversion of a step is a chain of shared-memory round trips
+// and a proxy fence; with one group the router took 29.8 us between its events
+// at N = 256, d = 7168, B = 256 and 37 us at N = 64, d = 2048, B = 8192, with
+// two 26.4 and 32 us),
+// warps 10-13 drain the TMEM buffers.  Every mbarrier wait is bounded; every thread reaches both
 // cluster barriers, so no CTA of a cluster can be left waiting on another.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -47,7 +51,8 @@ namespace {
 
 using namespace ptx;
 
-constexpr int kThreads = 320;
+constexpr int kThreads = 448;
+constexpr int kConvGroups = 2;                 // groups of four converter warps, taking turns
 constexpr int kBM = 128;                       // tokens per tile (MMA M)
 constexpr int kBK = 64;                        // K per stage
 constexpr int kXBytes = kBM * kBK * 2;         // 16 KB of x per stage
@@ -198,12 +203,12 @@ __global__ void __launch_bounds__(kThreads, 1) router_tc_kernel(const __grid_con
         mbar_wait(drain_bar, 0, kWaitNs, &no_abort);
       }
     }
-  } else if (warp < 6) {
+  } else if (warp < 2 + 4 * kConvGroups) {
     // ------------------------------------------------ weight planes
-    const int cw = warp - 2;
-    int stage = 0;
-    uint32_t phase = 0;
-    for (int kk = k_begin; kk < k_end; ++kk) {
+    const int cw = (warp - 2) & 3, group = (warp - 2) >> 2;
+    int stage = group % stages;
+    uint32_t phase = static_cast<uint32_t>(group / stages) & 1u;
+    for (int kk = k_begin + group; kk < k_end; kk += kConvGroups) {
       if (!mbar_wait(full_bar(stage), phase, kWaitNs, abort_flag)) {
         *abort_flag = 1;
         break;
@@ -230,8 +235,9 @@ __global__ void __launch_bounds__(kThreads, 1) router_tc_kernel(const __grid_con
       }
       fence_proxy_async_smem();
       mbar_arrive(conv_bar(stage));
-      if (++stage == stages) {
-        stage = 0;
+      stage += kConvGroups;
+      if (stage >= stages) {
+        stage -= stages;
         phase ^= 1u;
       }
     }
@@ -354,7 +360,7 @@ int cluster_cap(int nt, int S) {
 
 // Experts per tile (nt) and CTAs per cluster (S).  A CTA's time is a fixed
 // part (first loads, pipeline drain, cluster barriers, reduction: about
-// 6 us) plus about 0.55 us per K step of 64 whatever nt is (the round trip
+// 6 us) plus about 0.3 us per K step of 64 whatever nt is (the round trip
 // of a stage through TMA, plane conversion and MMA), so the shape with the
 // fewest K steps per CTA wins, among those whose clusters the device runs
 // at once; then the larger grid, then the fewer bytes per CTA.
