@@ -19,8 +19,10 @@
 // experts, B = 8192 (1365 tokens an expert) 1479 -> 735 us (gate/up 829 -> 340
 // us, 1.6 PFLOP/s; down 436 -> 212 us, which also writes 537 MB of fp32 rows);
 // d = 2048, F = 768, 128 experts, B = 2048 (128 tokens) 416 -> 310 us.  Four
-// pipeline stages of one K block instead of six cost 5 %, tiles dealt expert
-// by expert to all pairs (one row block at a time) 19 %.
+// pipeline stages instead of six cost 5 %, tiles dealt expert by expert to all
+// pairs (one row block at a time) 19 %.  With the loads left out the MMAs and
+// the epilogue of the first case's gate/up phase take 254 us (2.2 PFLOP/s), of
+// the second's 68 us (155 us with the loads, which stream 805 MB).
 //
 // Unit: (tile of up to 256 tokens of one expert, block of weight rows).  The
 // weights are the MMA's M = 256 rows, 128 in each CTA; the tokens are its N
@@ -55,14 +57,9 @@ using namespace ptx;
 constexpr int kBK = 64;                        // bf16 per K step (one 128-byte swizzle row)
 constexpr int kEpiWarps = 12;
 constexpr int kThreads = 64 + 32 * kEpiWarps;
-constexpr int kABytes = 128 * kBK * 2;         // this CTA's weight rows of a K block: 16 KB
-constexpr int kBlockBytes = 2 * kABytes;       // and up to 128 tokens
-// K blocks per pipeline stage (d and F are multiples of 128).  Two: a stage's
-// commit and wait cost the tensor cores about 57 ns (with the loads left out,
-// gate/up at B = 8192, N = 64, |S| = 48: 330 us with one block, 274 us with two).
-constexpr int kSub = 2;
-constexpr int kStages = 6 / kSub;
-constexpr int kStageBytes = kSub * kBlockBytes;
+constexpr int kABytes = 128 * kBK * 2;         // this CTA's weight rows of a step: 16 KB
+constexpr int kStageBytes = 2 * kABytes;       // and up to 128 tokens
+constexpr int kStages = 6;
 constexpr int kAccCols = 256;                  // TMEM columns per accumulator
 constexpr int kBarOffset = kStages * kStageBytes;
 constexpr int kSmemBytes = kBarOffset + 256 + 1024;   // + barriers + alignment slack
@@ -113,7 +110,7 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_pair_kernel(const __grid_cons
   const uint32_t rank = cluster_ctarank();
   const int t0 = __ldcg(&p.meta->ffn_t0), n_rt = __ldcg(&p.meta->ffn_t1) - t0;
   const int s0 = __ldcg(&p.meta->ffn_s0), n_tiles = n_rt + __ldcg(&p.meta->ffn_s1) - s0;
-  const int MB = kGateUp ? p.M / 128 : (p.M + 255) / 256, KI = p.K / kBK, KS = KI / kSub;
+  const int MB = kGateUp ? p.M / 128 : (p.M + 255) / 256, KI = p.K / kBK;
   const int n_units = n_tiles * MB;
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
   if (pair >= n_units) {  // both CTAs of the pair
@@ -171,9 +168,8 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_pair_kernel(const __grid_cons
   };
   const uint32_t full0 = map_to_rank(full_bar(0), 0);
 
-  // This CTA's operands of K block kk into sub-block i of a stage.
-  auto load_a = [&](const Unit &t, int kk, int stage, int i) {
-    const uint32_t dst = sbase + stage * kStageBytes + i * kBlockBytes, bar = full0 + 8u * stage;
+  auto load_a = [&](const Unit &t, int kk, int stage) {
+    const uint32_t dst = sbase + stage * kStageBytes, bar = full0 + 8u * stage;
     const CUtensorMap *m = t.routed ? p.tmA : p.tmS;
     if (kGateUp) {
       if (p.packed) {
@@ -194,14 +190,14 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_pair_kernel(const __grid_cons
         tma_load_2d_pair(dst, m, bar, kk * kBK, t.expert * p.M + mt * 128);
     }
   };
-  auto load_b = [&](const Unit &t, int kk, int stage, int i) {
+  auto load_b = [&](const Unit &t, int kk, int stage) {
     const int half = t.n_mma / 2;
-    tma_load_2d_pair(sbase + stage * kStageBytes + i * kBlockBytes + kABytes, &p.tmB[half / 16 - 1], full0 + 8u * stage,
+    tma_load_2d_pair(sbase + stage * kStageBytes + kABytes, &p.tmB[half / 16 - 1], full0 + 8u * stage,
                      kk * kBK, t.row0 + static_cast<int>(rank) * half);
   };
-  // Bytes that both CTAs bring in for one stage.
+  // Bytes that both CTAs bring in for one step.
   auto step_bytes = [&](const Unit &t) {
-    return kSub * static_cast<uint32_t>((rows_of(t, 1) ? 2 : 1) * kABytes + t.n_mma * kBK * 2);
+    return static_cast<uint32_t>((rows_of(t, 1) ? 2 : 1) * kABytes + t.n_mma * kBK * 2);
   };
   auto fail = [&]() {
     atomicMax(&p.meta->status, XS_DEV_TIMEOUT);
@@ -210,17 +206,19 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_pair_kernel(const __grid_cons
       st_cluster_u32(map_to_rank(smem_u32(const_cast<int *>(abort_flag)), r), 1u);
   };
 
-  const bool producer = warp == 0 && lane == 0;
   const int n_mine = (n_units - pair + n_pairs - 1) / n_pairs;
-  const long long steps = static_cast<long long>(n_mine) * KS;
+  const long long steps = static_cast<long long>(n_mine) * KI;
   const int n_pre = steps < kStages ? static_cast<int>(steps) : kStages;
-  if (producer) {
+  if (warp == 0) {
     // Every stage is free at the start: its weights do not wait for the kernel before.
     Unit t = unit_at(pair, true);
     for (int i = 0, kk = 0, u = pair; i < n_pre; ++i) {
-      if (rank == 0) mbar_arrive_expect_tx(full_bar(i), step_bytes(t));
-      for (int j = 0; j < kSub; ++j) load_a(t, kk * kSub + j, i, j);
-      if (++kk == KS && i + 1 < n_pre) {
+      if (elect_one()) {
+        if (rank == 0) mbar_arrive_expect_tx(full_bar(i), step_bytes(t));
+        load_a(t, kk, i);
+      }
+      __syncwarp();
+      if (++kk == KI && i + 1 < n_pre) {
         kk = 0;
         u += n_pairs;
         t = unit_at(u, true);
@@ -232,89 +230,89 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_pair_kernel(const __grid_cons
 
   if (warp == 0) {
     // ------------------------------------------------ TMA producer
-    if (lane == 0) {
-      int stage = 0, i = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int u = pair; ok && u < n_units; u += n_pairs) {
-        const Unit t = unit_at(u, false);
-        const uint32_t bytes = step_bytes(t);
-        for (int kk = 0; kk < KS; ++kk, ++i) {
-          if (i >= n_pre) {
-            if (!mbar_wait(empty_bar(stage), phase ^ 1u, kWaitNs, abort_flag)) {
-              ok = false;
-              break;
-            }
-            if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), bytes);
-            for (int j = 0; j < kSub; ++j) load_a(t, kk * kSub + j, stage, j);
-          }
-          for (int j = 0; j < kSub; ++j) load_b(t, kk * kSub + j, stage, j);
-          if (++stage == kStages) {
-            stage = 0;
-            phase ^= 1u;
-          }
+    int stage = 0, i = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int u = pair; ok && u < n_units; u += n_pairs) {
+      const Unit t = unit_at(u, false);
+      const uint32_t bytes = step_bytes(t);
+      for (int kk = 0; kk < KI; ++kk, ++i) {
+        if (i >= n_pre) {
+          ok = __all_sync(0xffffffffu, mbar_wait(empty_bar(stage), phase ^ 1u, kWaitNs, abort_flag));
+          if (!ok) break;
         }
-      }
-      // The last MMAs have read every stage, and this CTA got every signal that
-      // is sent to it.
-      for (int j = 0; ok && j < kStages; ++j) {
-        ok = mbar_wait(empty_bar(stage), phase ^ 1u, kWaitNs, abort_flag);
+        if (elect_one()) {
+          if (i >= n_pre) {
+            if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), bytes);
+            load_a(t, kk, stage);
+          }
+          load_b(t, kk, stage);
+        }
+        __syncwarp();
         if (++stage == kStages) {
           stage = 0;
           phase ^= 1u;
         }
       }
-      if (!ok) {
-        fail();
-        // Copies may be in flight whose barrier no longer completes: they land
-        // in microseconds; stay for two milliseconds.
-        const uint64_t t_end = globaltimer() + 2000000ull;
-        while (globaltimer() < t_end) __nanosleep(1000);
+    }
+    // The last MMAs have read every stage, and this CTA got every signal that
+    // is sent to it.
+    for (int j = 0; ok && j < kStages; ++j) {
+      ok = __all_sync(0xffffffffu, mbar_wait(empty_bar(stage), phase ^ 1u, kWaitNs, abort_flag));
+      if (++stage == kStages) {
+        stage = 0;
+        phase ^= 1u;
       }
+    }
+    if (!ok) {
+      if (lane == 0) fail();
+      // Copies may be in flight whose barrier no longer completes: they land
+      // in microseconds; stay for two milliseconds.
+      const uint64_t t_end = globaltimer() + 2000000ull;
+      while (globaltimer() < t_end) __nanosleep(1000);
     }
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer (rank 0)
-    if (rank == 0 && lane == 0) {
-      const uint64_t desc0 = sw128_desc(sbase);  // stages and K blocks are added to its address field
+    if (rank == 0) {
+      // Stages and K blocks are added to the descriptor's address field.
+      const uint64_t desc0 = sw128_desc(__shfl_sync(0xffffffffu, sbase, 0));
+      const uint32_t acc0 = __shfl_sync(0xffffffffu, tmem, 0);
       int stage = 0, seq = 0;
       uint32_t phase = 0;
       bool ok = true;
       for (int u = pair; ok && u < n_units; u += n_pairs, ++seq) {
         const Unit t = unit_at(u, false);
-        const uint32_t idesc = idesc_bf16(256, t.n_mma);
+        const uint32_t idesc = __shfl_sync(0xffffffffu, idesc_bf16(256, t.n_mma), 0);
         const int buf = seq & 1;
-        if (!mbar_wait(accempty_bar(buf), ((seq >> 1) & 1u) ^ 1u, kWaitNs, abort_flag)) {
-          ok = false;
-          break;
-        }
+        ok = __all_sync(0xffffffffu, mbar_wait(accempty_bar(buf), ((seq >> 1) & 1u) ^ 1u, kWaitNs, abort_flag));
+        if (!ok) break;
         tc_fence_after();
-        const uint32_t d0 = tmem + buf * kAccCols;
-        for (int kk = 0; kk < KS; ++kk) {
-          if (!mbar_wait(full_bar(stage), phase, kWaitNs, abort_flag)) {
-            ok = false;
-            break;
-          }
+        const uint32_t d0 = acc0 + buf * kAccCols;
+        for (int kk = 0; kk < KI; ++kk) {
+          ok = __all_sync(0xffffffffu, mbar_wait(full_bar(stage), phase, kWaitNs, abort_flag));
+          if (!ok) break;
           tc_fence_after();
           const uint64_t da = desc0 + static_cast<uint64_t>(stage * (kStageBytes >> 4));
-#pragma unroll
-          for (int j = 0; j < kSub; ++j)
+          if (elect_one()) {
 #pragma unroll
             for (int ks = 0; ks < kBK / 16; ++ks) {
-              const uint64_t a = da + static_cast<uint64_t>((j * kBlockBytes + ks * 32) >> 4);
-              mma_bf16_pair(d0, a, a + (kABytes >> 4), idesc, (kk > 0 || j > 0 || ks > 0) ? 1u : 0u);
+              const uint64_t a = da + static_cast<uint64_t>((ks * 32) >> 4);
+              mma_bf16_pair(d0, a, a + (kABytes >> 4), idesc, (kk > 0 || ks > 0) ? 1u : 0u);
             }
-          mma_commit_pair(empty_bar(stage));
+            mma_commit_pair(empty_bar(stage));
+            if (kk + 1 == KI) mma_commit_pair(accfull_bar(buf));
+          }
+          __syncwarp();
           if (++stage == kStages) {
             stage = 0;
             phase ^= 1u;
           }
         }
-        if (ok) mma_commit_pair(accfull_bar(buf));
       }
-      if (!ok) fail();
+      if (!ok && lane == 0) fail();
       // All issued MMAs done before TMEM is released.
+      if (elect_one()) mma_commit_pair_local(drain_bar);
       volatile int no_abort = 0;
-      mma_commit_pair_local(drain_bar);
       mbar_wait(drain_bar, 0, kWaitNs, &no_abort);
     }
   } else {

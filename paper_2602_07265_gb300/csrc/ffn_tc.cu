@@ -231,7 +231,6 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_tc_kernel(const __grid_consta
       if (kGateUp) tma_load_2d(sA + kTileBytes, r.mA1, bar, kk * kBK, r.arow, pol);
     }
   };
-  const bool producer = warp == 0 && lane == 0;
   const int n_pre = (it_end - it_begin) < C::kStages ? static_cast<int>(it_end - it_begin) : C::kStages;
   // The CTA's steps as segments (unit u, steps [k0, k1) of it), in the order
   // all three roles process them: first the piece of the last unit that the
@@ -287,7 +286,7 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_tc_kernel(const __grid_consta
     }
   };
   uint64_t pol_w = 0, pol_x = 0;
-  if (producer) {
+  if (warp == 0) {
     // Every stage is free at the start: fill the ring with weights and warm L2
     // with the weights that follow.
     pol_w = policy_evict_first();
@@ -296,15 +295,20 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_tc_kernel(const __grid_consta
     Src r{};
     for (int i = 0; i < n_pre; ++i, advance(c)) {
       source(c, r, true);
-      mbar_arrive_expect_tx(full_bar(i), r.tx);
-      load_weights(r, c.kk, sbase + i * C::kStageBytes, full_bar(i), pol_w);
+      if (elect_one()) {
+        mbar_arrive_expect_tx(full_bar(i), r.tx);
+        load_weights(r, c.kk, sbase + i * C::kStageBytes, full_bar(i), pol_w);
+      }
+      __syncwarp();
     }
     if (p.pk) {
       const long long n_pf = C::kL2Prefetch / (C::kNumA * kTileBytes);
       for (long long it = it_begin + n_pre; it < it_end && it < it_begin + n_pre + n_pf; ++it, advance(c)) {
         source(c, r, true);
-        bulk_prefetch_l2(r.pblk + static_cast<size_t>(c.kk) * (C::kNumA * kTileBytes),
-                         C::kNumA * kTileBytes);
+        if (elect_one())
+          bulk_prefetch_l2(r.pblk + static_cast<size_t>(c.kk) * (C::kNumA * kTileBytes),
+                           C::kNumA * kTileBytes);
+        __syncwarp();
       }
     }
   }
@@ -313,77 +317,75 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_tc_kernel(const __grid_consta
 
   if (warp == 0) {
     // ------------------------------------------------ TMA producer
-    if (lane == 0) {
-      uint32_t issued_mask = 0, issued_phase = 0;
-      Cursor c = c_begin;
-      Src r{};
-      // Token operand of the stages filled above.
-      for (int i = 0; i < n_pre; ++i, advance(c)) {
-        source(c, r, false);
+    uint32_t issued_mask = 0, issued_phase = 0;
+    Cursor c = c_begin;
+    Src r{};
+    // Token operand of the stages filled above.
+    for (int i = 0; i < n_pre; ++i, advance(c)) {
+      source(c, r, false);
+      if (elect_one())
         tma_load_2d(sbase + i * C::kStageBytes + C::kNumA * kTileBytes, &p.tmB[r.bsel], full_bar(i),
                     c.kk * kBK, r.row0, pol_x);
-        issued_mask |= 1u << i;
-      }
-      int stage = static_cast<int>(n_pre % C::kStages);
-      uint32_t phase = n_pre == C::kStages ? 1u : 0u;
-      bool ok = true;
-      for (long long it = it_begin + n_pre; it < it_end; ++it, advance(c)) {
-        source(c, r, false);
-        const int kk = c.kk;
-        if (!mbar_wait(empty_bar(stage), phase ^ 1u, kWaitNs, abort_flag)) {
-          ok = false;
-          break;
-        }
+      __syncwarp();
+      issued_mask |= 1u << i;
+    }
+    int stage = static_cast<int>(n_pre % C::kStages);
+    uint32_t phase = n_pre == C::kStages ? 1u : 0u;
+    bool ok = true;
+    for (long long it = it_begin + n_pre; it < it_end; ++it, advance(c)) {
+      source(c, r, false);
+      const int kk = c.kk;
+      ok = __all_sync(0xffffffffu, mbar_wait(empty_bar(stage), phase ^ 1u, kWaitNs, abort_flag));
+      if (!ok) break;
+      if (elect_one()) {
         const uint32_t sA = sbase + stage * C::kStageBytes;
         mbar_arrive_expect_tx(full_bar(stage), r.tx);
         load_weights(r, kk, sA, full_bar(stage), pol_w);
         tma_load_2d(sA + C::kNumA * kTileBytes, &p.tmB[r.bsel], full_bar(stage), kk * kBK, r.row0, pol_x);
-        issued_mask |= 1u << stage;
-        issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
-        if (++stage == C::kStages) {
-          stage = 0;
-          phase ^= 1u;
-        }
       }
-      if (!ok) {
-        set_status(p, XS_DEV_TIMEOUT);
-        *abort_flag = 1;
+      __syncwarp();
+      issued_mask |= 1u << stage;
+      issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
+      if (++stage == C::kStages) {
+        stage = 0;
+        phase ^= 1u;
       }
-      // Never leave with copies in flight: wait (bounded) for the last load of every stage.
-      volatile int no_abort = 0;
-      for (int s = 0; s < C::kStages; ++s)
-        if ((issued_mask >> s) & 1u) mbar_wait(full_bar(s), (issued_phase >> s) & 1u, kWaitNs, &no_abort);
     }
+    if (!ok && lane == 0) {
+      set_status(p, XS_DEV_TIMEOUT);
+      *abort_flag = 1;
+    }
+    // Never leave with copies in flight: wait (bounded) for the last load of every stage.
+    volatile int no_abort = 0;
+    for (int s = 0; s < C::kStages; ++s)
+      if ((issued_mask >> s) & 1u) mbar_wait(full_bar(s), (issued_phase >> s) & 1u, kWaitNs, &no_abort);
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      int segi = 0;
-      bool ok = true, any = false;
-      for (; ok && segi < n_seg; ++segi) {
-        const Seg g = seg_at(segi);
-        const long long u = g.u;
-        const int k0 = g.k0, k1 = g.k1;
-        const Tile tl = p.tiles[wt.tile(static_cast<int>(u / MT))];
-        const int n_mma = ((tl.ntok + 15) / 16) * 16;
-        const uint32_t idesc = idesc_bf16(kBM, n_mma);
-        const int buf = segi & 1;
-        const uint32_t use = static_cast<uint32_t>(segi >> 1);
-        if (!mbar_wait(accempty_bar(buf), (use & 1u) ^ 1u, kWaitNs, abort_flag)) {
-          ok = false;
-          break;
-        }
+    const uint32_t base = __shfl_sync(0xffffffffu, sbase, 0), acc0 = __shfl_sync(0xffffffffu, tmem, 0);
+    int stage = 0;
+    uint32_t phase = 0;
+    int segi = 0;
+    bool ok = true, any = false;
+    for (; ok && segi < n_seg; ++segi) {
+      const Seg g = seg_at(segi);
+      const long long u = g.u;
+      const int k0 = g.k0, k1 = g.k1;
+      const Tile tl = p.tiles[wt.tile(static_cast<int>(u / MT))];
+      const int n_mma = ((tl.ntok + 15) / 16) * 16;
+      const uint32_t idesc = __shfl_sync(0xffffffffu, idesc_bf16(kBM, n_mma), 0);
+      const int buf = segi & 1;
+      const uint32_t use = static_cast<uint32_t>(segi >> 1);
+      ok = __all_sync(0xffffffffu, mbar_wait(accempty_bar(buf), (use & 1u) ^ 1u, kWaitNs, abort_flag));
+      if (!ok) break;
+      tc_fence_after();
+      const uint32_t d0 = acc0 + buf * C::kAccCols;
+      for (int kk = k0; kk < k1; ++kk) {
+        ok = __all_sync(0xffffffffu, mbar_wait(full_bar(stage), phase, kWaitNs, abort_flag));
+        if (!ok) break;
         tc_fence_after();
-        const uint32_t d0 = tmem + buf * C::kAccCols;
-        for (int kk = k0; kk < k1; ++kk) {
-          if (!mbar_wait(full_bar(stage), phase, kWaitNs, abort_flag)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t sA = sbase + stage * C::kStageBytes;
-          const uint32_t sB = sA + C::kNumA * kTileBytes;
+        const uint32_t sA = base + stage * C::kStageBytes;
+        const uint32_t sB = sA + C::kNumA * kTileBytes;
+        if (elect_one()) {
 #pragma unroll
           for (int ks = 0; ks < kBK / 16; ++ks) {
             const uint32_t acc = (kk > k0 || ks > 0) ? 1u : 0u;
@@ -391,25 +393,25 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_tc_kernel(const __grid_consta
             mma_bf16(d0, sw128_desc(sA + ks * 32), db, idesc, acc);
             if (kGateUp) mma_bf16(d0 + 128, sw128_desc(sA + kTileBytes + ks * 32), db, idesc, acc);
           }
-          any = true;
           mma_commit(empty_bar(stage));
-          if (++stage == C::kStages) {
-            stage = 0;
-            phase ^= 1u;
-          }
+          if (kk + 1 == k1) mma_commit(accfull_bar(buf));
         }
-        if (!ok) break;
-        mma_commit(accfull_bar(buf));
+        __syncwarp();
+        any = true;
+        if (++stage == C::kStages) {
+          stage = 0;
+          phase ^= 1u;
+        }
       }
-      if (!ok) {
-        set_status(p, XS_DEV_TIMEOUT);
-        *abort_flag = 1;
-      }
-      if (any) {  // all issued MMAs done before TMEM is released
-        volatile int no_abort = 0;
-        mma_commit(drain_bar);
-        mbar_wait(drain_bar, 0, kWaitNs, &no_abort);
-      }
+    }
+    if (!ok && lane == 0) {
+      set_status(p, XS_DEV_TIMEOUT);
+      *abort_flag = 1;
+    }
+    if (any) {  // all issued MMAs done before TMEM is released
+      volatile int no_abort = 0;
+      if (elect_one()) mma_commit(drain_bar);
+      mbar_wait(drain_bar, 0, kWaitNs, &no_abort);
     }
   } else {
     // ------------------------------------------------ epilogue (warps 2..5)

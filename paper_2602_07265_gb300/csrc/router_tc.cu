@@ -139,69 +139,73 @@ __global__ void __launch_bounds__(kThreads, 1) router_tc_kernel(const __grid_con
 
   if (warp == 0) {
     // ------------------------------------------------ TMA producer
-    if (lane == 0) {
-      const uint64_t pol = policy_evict_last();  // W_g and x are reread by other tiles
-      const uint32_t tx = kXBytes + kNt * kBK * 4;
-      int stage = 0;
-      uint32_t phase = 0, issued_mask = 0, issued_phase = 0;
-      for (int kk = k_begin; kk < k_end; ++kk) {
-        if (!mbar_wait(empty_bar(stage), phase ^ 1u, kWaitNs, abort_flag)) {
-          *abort_flag = 1;
-          break;
-        }
+    const uint64_t pol = policy_evict_last();  // W_g and x are reread by other tiles
+    const uint32_t tx = kXBytes + kNt * kBK * 4;
+    int stage = 0;
+    uint32_t phase = 0, issued_mask = 0, issued_phase = 0;
+    for (int kk = k_begin; kk < k_end; ++kk) {
+      if (!__all_sync(0xffffffffu, mbar_wait(empty_bar(stage), phase ^ 1u, kWaitNs, abort_flag))) {
+        *abort_flag = 1;
+        break;
+      }
+      if (elect_one()) {
         mbar_arrive_expect_tx(full_bar(stage), tx);
         tma_load_2d(x_s(stage), &p.tmX, full_bar(stage), kk * kBK, m0, pol);
         tma_load_2d(smem_u32(w_s(stage)), &p.tmW, full_bar(stage), kk * kBK, n0, pol);
-        issued_mask |= 1u << stage;
-        issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
-        if (++stage == stages) {
-          stage = 0;
-          phase ^= 1u;
-        }
       }
-      // Never leave with copies in flight: wait (bounded) for the last load of every stage.
-      volatile int no_abort = 0;
-      for (int s = 0; s < stages; ++s)
-        if ((issued_mask >> s) & 1u) mbar_wait(full_bar(s), (issued_phase >> s) & 1u, kWaitNs, &no_abort);
+      __syncwarp();
+      issued_mask |= 1u << stage;
+      issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
+      if (++stage == stages) {
+        stage = 0;
+        phase ^= 1u;
+      }
     }
+    // Never leave with copies in flight: wait (bounded) for the last load of every stage.
+    volatile int no_abort = 0;
+    for (int s = 0; s < stages; ++s)
+      if ((issued_mask >> s) & 1u) mbar_wait(full_bar(s), (issued_phase >> s) & 1u, kWaitNs, &no_abort);
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      const uint32_t idesc = idesc_bf16(kBM, kNt);
-      int stage = 0;
-      uint32_t phase = 0;
-      bool any = false;
-      for (int kk = k_begin; kk < k_end; ++kk) {
-        const int i = kk - k_begin, buf = i % kBufs;
-        const uint32_t use = static_cast<uint32_t>(i / kBufs);
-        if (!mbar_wait(conv_bar(stage), phase, kWaitNs, abort_flag) ||
-            !mbar_wait(acce_bar(buf), (use & 1u) ^ 1u, kWaitNs, abort_flag)) {
-          *abort_flag = 1;
-          break;
-        }
-        tc_fence_after();
-        const uint32_t d0 = tmem + static_cast<uint32_t>(buf * kNt);
+    const uint32_t idesc = idesc_bf16(kBM, kNt);
+    const uint32_t base = __shfl_sync(0xffffffffu, sbase, 0), acc0 = __shfl_sync(0xffffffffu, tmem, 0);
+    int stage = 0;
+    uint32_t phase = 0;
+    bool any = false;
+    for (int kk = k_begin; kk < k_end; ++kk) {
+      const int i = kk - k_begin, buf = i % kBufs;
+      const uint32_t use = static_cast<uint32_t>(i / kBufs);
+      const bool ready = mbar_wait(conv_bar(stage), phase, kWaitNs, abort_flag) &&
+                         mbar_wait(acce_bar(buf), (use & 1u) ^ 1u, kWaitNs, abort_flag);
+      if (!__all_sync(0xffffffffu, ready)) {
+        *abort_flag = 1;
+        break;
+      }
+      tc_fence_after();
+      const uint32_t d0 = acc0 + static_cast<uint32_t>(buf * kNt), xs = base + stage * sb;
+      if (elect_one()) {
 #pragma unroll
         for (int ks = 0; ks < kBK / 16; ++ks) {
-          const uint64_t da = sw128_desc(x_s(stage) + ks * 32);
+          const uint64_t da = sw128_desc(xs + ks * 32);
 #pragma unroll
           for (int pl = 0; pl < 3; ++pl)
-            mma_bf16(d0, da, sw128_desc(plane_s(stage, pl) + ks * 32), idesc,
+            mma_bf16(d0, da, sw128_desc(xs + kXBytes + kNt * kBK * 4 + pl * kNt * 128 + ks * 32), idesc,
                      (ks > 0 || pl > 0) ? 1u : 0u);
         }
-        any = true;
         mma_commit(empty_bar(stage));
         mma_commit(accf_bar(buf));
-        if (++stage == stages) {
-          stage = 0;
-          phase ^= 1u;
-        }
       }
-      if (any) {  // all issued MMAs done before TMEM is released
-        volatile int no_abort = 0;
-        mma_commit(drain_bar);
-        mbar_wait(drain_bar, 0, kWaitNs, &no_abort);
+      __syncwarp();
+      any = true;
+      if (++stage == stages) {
+        stage = 0;
+        phase ^= 1u;
       }
+    }
+    if (any) {  // all issued MMAs done before TMEM is released
+      volatile int no_abort = 0;
+      if (elect_one()) mma_commit(drain_bar);
+      mbar_wait(drain_bar, 0, kWaitNs, &no_abort);
     }
   } else if (warp < 2 + 4 * kConvGroups) {
     // ------------------------------------------------ weight planes
