@@ -322,7 +322,7 @@ int xs::forward_impl(const FwdCall &c, FwdStep step) {
   // the selected set is known (packed weights, without expert parallelism).
   GatherPf pf;
   std::memset(&pf, 0, sizeof(pf));
-  if (packed && !ep && !ffn_pairs) {
+  if (packed && !ep) {
     pf.ready = a.done + 3;
     pf.mask = a.mask;
     pf.pk = static_cast<const uint8_t *>(c.P_gate_up);
@@ -332,9 +332,11 @@ int xs::forward_impl(const FwdCall &c, FwdStep step) {
     pf.stage_bytes = 2 * 128 * 64 * 2;
     pf.grid = sms;
     pf.max_used = B * k;
+    pf.linear = ffn_pairs;
     // A refinement kernel of its own (more than kFuseChunks chunks) leaves
     // a longer window before the gate/up kernel: twice the warm-up.
     pf.pf_bytes = (B + kChunk - 1) / kChunk > kFuseChunks ? 2 * kGatherPrefetchBytes : kGatherPrefetchBytes;
+    if (ffn_pairs) pf.pf_bytes = kPairWarmBytes;
   }
   if (launch_gather(c.x, a, const_cast<uint16_t *>(f.xp), ep ? f.out : nullptr, d, sms, pf, s) !=
           cudaSuccess ||

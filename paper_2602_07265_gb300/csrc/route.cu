@@ -1534,6 +1534,20 @@ __device__ void warm_gate_up(const GatherPf &g, int32_t *s_sel, int *s_n) {
   const int nS = *s_n;
   if (nS <= 0 || nS > g.max_used) return;
   const long long KI = g.KI, I = static_cast<long long>(nS) * g.MT * KI;
+  if (g.linear) {
+    // ffn_pair.cu deals the units out in expert order: the first bytes of the
+    // selected experts in turn, whole blocks (an expert's are contiguous).
+    const long long n = min(I, static_cast<long long>(g.pf_bytes / g.stage_bytes));
+    const long long per = static_cast<long long>(g.MT) * KI;
+    for (long long i = blockIdx.x + static_cast<long long>(tid) * kGatherWarmBlocks; i < n;
+         i += static_cast<long long>(blockDim.x) * kGatherWarmBlocks) {
+      const uint8_t *blk = g.pk + (s_sel[i / per] * per + i % per) * static_cast<size_t>(g.stage_bytes);
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(reinterpret_cast<uint64_t>(blk)),
+                   "r"(g.stage_bytes)
+                   : "memory");
+    }
+    return;
+  }
   const int G = ffn_ctas(static_cast<long long>(nS) * g.MT, g.KI, g.grid);  // gate/up CTAs
   const int n_steps = g.pf_bytes / g.stage_bytes;
   const int nb = gridDim.x < kGatherWarmBlocks ? static_cast<int>(gridDim.x) : kGatherWarmBlocks;

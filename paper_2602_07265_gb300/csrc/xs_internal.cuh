@@ -54,6 +54,10 @@ constexpr int kScoreRowBytes = 190 * 1024;   // score rows of a selection CTA at
 constexpr int kFuseChunks = 2;               // up to this many chunks the selection CTA also refines
 constexpr int kMaxShared = 8;                // shared experts
 constexpr int kGatherPrefetchBytes = 256 * 1024;  // L2 warm-up per gate/up CTA (packed weights)
+// The same for the CTA-pair kernel, in total: layer forward at N = 64, d = 2048,
+// F = 1024, B = 512 without, 32, 64 and 96 MB 170.4, 168.3, 166.4, 166.9 us; no
+// difference from B = 2048 on.
+constexpr int kPairWarmBytes = 64 * 1024 * 1024;
 constexpr int kGatherWarmBlocks = 32;              // gather blocks that issue the warm-up
 
 // CTAs an FFN kernel splits its U units (a token tile x 128 weight rows, KI
@@ -203,6 +207,7 @@ struct GatherPf {
   int stage_bytes;        // packed bytes per step (gate and up tiles)
   int grid;               // the gate/up kernel's grid
   int pf_bytes;           // bytes per gate/up CTA to prefetch
+  int linear;             // ffn_pair.cu's order; pf_bytes is then the total
   int max_used;           // at most this many experts get a token (the batch's pairs)
 };
 // Places the pairs of the routing `a` and gathers the token rows of this
