@@ -532,7 +532,7 @@ __device__ __forceinline__ void write_tiles(Tile *tiles, int tile0, int e, int r
     tl.expert = e;
     tl.row0 = row0 + lo;
     tl.ntok = hi - lo;
-    tl.pad = 0;
+    tl.single = n == 1;
     tiles[tile0 + i] = tl;
   }
 }
@@ -735,7 +735,7 @@ __device__ void build_permutation_small(const RouteArgs &a, uint32_t *s_tm0, uin
           tl.expert = e;
           tl.row0 = row;
           tl.ntok = c;
-          tl.pad = 0;
+          tl.single = 1;
           a.tiles[tile] = tl;
         }
       }
@@ -750,7 +750,7 @@ __device__ void build_permutation_small(const RouteArgs &a, uint32_t *s_tm0, uin
       tl.expert = N + j;
       tl.row0 = tot_rows + j * B;
       tl.ntok = B;
-      tl.pad = 0;
+      tl.single = 1;
       a.tiles[tot_tiles + j] = tl;
     }
     if (lane == 0) {

@@ -82,12 +82,13 @@ __host__ __device__ inline int ffn_ctas(long long U, int KI, int grid) {
 
 // Batches with at least this many routed pairs per expert that can be
 // selected take the CTA-pair FFN kernels (ffn_pair.cu).
-// Both sides on GB300, plain top-k, whole layer, ffn_tc.cu | ffn_pair.cu at 48,
-// 64, 96 and 128 pairs an expert: N = 64, d = 2048, F = 1024: 168 | 173, 179 |
-// 179, 207 | 191, 286 | 205 us; N = 128, F = 768: 248 | 257, 264 | 265 us at 48
-// and 64, 416 | 319 us at 128.  Below, the weights' stream is the bound and
-// ffn_tc.cu splits it over the SMs without a remainder.
-constexpr int kPairMinTok = 64;
+// Both sides on GB300, plain top-k, whole layer, ffn_tc.cu | ffn_pair.cu at 8,
+// 16, 24, 32, 48 and 64 pairs an expert: N = 64, d = 2048, F = 1024: 142.4 |
+// 145.4, 146.5 | 144.9, 149.5 | 146.8, 152.3 | 149.5, 161.1 | 150.6, 171.9 |
+// 156.7 us; N = 128, F = 768 from 16 on: 208.4 | 212.5, 213.4 | 213.5, 224.3 |
+// 218.9, 233.9 | 228.3, 252.1 | 237.0 us.  Below, ffn_tc.cu's split of the
+// weight stream without a remainder wins.
+constexpr int kPairMinTok = 24;
 
 // One FFN work tile: up to kTileTok (kPairTok) consecutive rows of the permuted pair
 // list, all routed to `expert`.  Experts N .. N + n_shared - 1 are the shared
@@ -97,7 +98,7 @@ struct Tile {
   int32_t expert;
   int32_t row0;
   int32_t ntok;
-  int32_t pad;
+  int32_t single;   // the expert's only tile
 };
 
 // Device-side facts of one call, written by the routing kernel and read by
