@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_pair_kernel(const __grid_cons
     mbar_init(drain_bar, 1);
     *abort_flag = 0;
     fence_mbar_init();
-    for (int i = 0; i < 8; ++i) prefetch_tmap(&p.tmB[i]);
+    prefetch_tmap(&p.tmB[0]);
     prefetch_tmap(&p.tmA[0]);
   }
   if (warp == 1) {
@@ -325,7 +325,9 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_pair_kernel(const __grid_cons
   } else {
     // ------------------------------------------------ epilogue
     const int q = warp & 3;                  // TMEM lane quarter of this warp
+    const int row = q * 32 + lane;           // this thread's accumulator row
     const int first = (warp - 2) / 4 * 32;   // its first column; every other 8 kEpiWarps
+    constexpr int kStep = 8 * kEpiWarps;
     const uint32_t accempty0 = map_to_rank(accempty_bar(0), 0);
     int seq = 0;
     for (int u = pair; u < n_units; u += n_pairs, ++seq) {
@@ -338,47 +340,42 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_pair_kernel(const __grid_cons
       __syncwarp();
       tc_fence_after();
       const uint32_t tacc = tmem + (static_cast<uint32_t>(q * 32) << 16) + buf * kAccCols;
+      const int n_cols = rows_of(t, rank) ? t.n_mma : 0;   // columns this CTA finishes
       // The accumulator is free once this warp's last columns are in registers.
-      auto loaded = [&](int c0) {
-        if (c0 + 8 * kEpiWarps < t.n_mma) return;
+      auto release = [&]() {
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster(accempty0 + 8u * buf);
       };
-      if (first >= t.n_mma || !rows_of(t, rank)) {
-        loaded(t.n_mma);
-        continue;
-      }
-      if (kGateUp) {
-        // Lanes 0-15 hold the gate rows of 16 hidden units, lanes 16-31 their
-        // up rows; of every two tokens each half finishes one.
-        const bool hi = lane >= 16;
-        const int f = t.mb * 128 + static_cast<int>(rank) * 64 + q * 16 + (lane & 15);
-        uint16_t *dst = p.act_out + static_cast<size_t>(t.row0 + (hi ? 1 : 0)) * p.M + f;
-        for (int c0 = first; c0 < t.n_mma; c0 += 8 * kEpiWarps) {
-          float v[32];
-          tmem_ld32(tacc + c0, v);
-          loaded(c0);
+      // Finishes columns [c0, c0 + 32): this thread's row of them in v.
+      auto emit = [&](int c0, const float (&v)[32]) {
+        if (kGateUp) {
+          // Lanes 0-15 hold the gate rows of 16 hidden units, lanes 16-31 their
+          // up rows; of every two tokens each half finishes one.
+          const bool up_half = lane >= 16;
+          const int f = t.mb * 128 + static_cast<int>(rank) * 64 + q * 16 + (lane & 15);
+          uint16_t *dst = p.act_out + static_cast<size_t>(t.row0 + c0 + (up_half ? 1 : 0)) * p.M + f;
 #pragma unroll
           for (int j = 0; j < 32; j += 2) {
-            const float other = __shfl_xor_sync(0xffffffffu, hi ? v[j] : v[j + 1], 16);
-            const float g = hi ? other : v[j], up = hi ? v[j + 1] : other;
-            const __nv_bfloat16 h = __float2bfloat16_rn(silu(g) * up);
-            if (c0 + j + (hi ? 1 : 0) < t.ntok)
-              dst[static_cast<size_t>(c0 + j) * p.M] = *reinterpret_cast<const uint16_t *>(&h);
+            const float other = __shfl_xor_sync(0xffffffffu, up_half ? v[j] : v[j + 1], 16);
+            const float gate = up_half ? other : v[j], up = up_half ? v[j + 1] : other;
+            const __nv_bfloat16 h = __float2bfloat16_rn(silu(gate) * up);
+            if (c0 + j + (up_half ? 1 : 0) < t.ntok)
+              dst[static_cast<size_t>(j) * p.M] = *reinterpret_cast<const uint16_t *>(&h);
           }
-        }
-      } else {
-        const int row = t.mb * 256 + static_cast<int>(rank) * 128 + q * 32 + lane;
-        float *dst = p.out + static_cast<size_t>(t.row0) * p.M + row;
-        for (int c0 = first; c0 < t.n_mma; c0 += 8 * kEpiWarps) {
-          float v[32];
-          tmem_ld32(tacc + c0, v);
-          loaded(c0);
+        } else {
+          float *dst = p.out + static_cast<size_t>(t.row0 + c0) * p.M + t.mb * 256 + static_cast<int>(rank) * 128 + row;
 #pragma unroll
           for (int j = 0; j < 32; ++j)
-            if (c0 + j < t.ntok) dst[static_cast<size_t>(c0 + j) * p.M] = v[j];
+            if (c0 + j < t.ntok) dst[static_cast<size_t>(j) * p.M] = v[j];
         }
+      };
+      if (first >= n_cols) release();
+      for (int c0 = first; c0 < n_cols; c0 += kStep) {
+        float v[32];
+        tmem_ld32(tacc + c0, v);
+        if (c0 + kStep >= n_cols) release();
+        emit(c0, v);
       }
     }
   }
