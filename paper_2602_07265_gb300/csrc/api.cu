@@ -101,6 +101,22 @@ RouteArgs route_args(const Plan &pl, void *ws, int B, int N, int k, int budget, 
   return a;
 }
 
+// At most this many experts can be selected (budgets add to the
+// warm-up sets).
+int max_selected(const RouteArgs &a) {
+  const long long warm = static_cast<long long>(a.B) * a.k0;
+  long long n = a.N;
+  if (a.mode == XS_MODE_BATCH) {
+    n = warm + a.budget;
+  } else if (a.mode == XS_MODE_HIER) {
+    n = warm + static_cast<long long>(a.B / a.T) * a.m_r + a.budget;
+  } else if (a.mode == XS_MODE_GROUP) {
+    const long long rounds = static_cast<long long>(a.m_g) * a.G + a.G - 1;
+    n = warm > rounds ? warm : rounds;
+  }
+  return static_cast<int>(n < a.N ? n : a.N);
+}
+
 }  // namespace
 
 Plan make_plan(int B, int N, int k, int d, int F, bool with_ffn, int n_sms, int n_shared) {
@@ -256,9 +272,7 @@ int xs::forward_impl(const FwdCall &c, FwdStep step) {
   a.zero_words = at<int32_t>(workspace, pl.ffn_cnt);
   a.zero_count = (int)ffn_cnt_words(pl.max_tiles, B, d, F);
   a.n_shared = n_shared;
-  // At most this many experts can be selected (BATCH: warm-up and budget).
-  const long long sel_max = c.mode == XS_MODE_BATCH ? static_cast<long long>(B) * c.prm->k0 + c.budget : N;
-  const bool ffn_pairs = ffn_use_pairs(static_cast<long long>(B) * k, static_cast<int>(sel_max < N ? sel_max : N));
+  const bool ffn_pairs = ffn_use_pairs(static_cast<long long>(B) * k, max_selected(a), d, F);
   if (ffn_pairs) a.tile_tok = kPairTok;
 
   FfnArgs f;

@@ -501,8 +501,19 @@ cudaError_t launch_phase(const FfnArgs &a, cudaStream_t s) {
 
 }  // namespace
 
-bool ffn_use_pairs(long long pairs, int experts) {
-  return pairs >= static_cast<long long>(kPairMinTok) * experts && resident_pairs() > 0;
+bool ffn_use_pairs(long long pairs, int experts, int d, int F) {
+  const int P = resident_pairs();
+  if (P <= 0 || experts <= 0) return false;
+  if (pairs >= static_cast<long long>(kPairMinTok) * experts) return true;
+  if (pairs < static_cast<long long>(kPairFewTok) * experts &&
+      pairs * d < static_cast<long long>(kPairWork) * experts)
+    return false;
+  // Rounds that the whole units take, against the time their work would fill.
+  auto idles = [&](double blocks, int units) {
+    const long long rounds = (static_cast<long long>(experts) * units + P - 1) / P;
+    return static_cast<double>(rounds) * P > experts * blocks * (1.0 + kPairIdle);
+  };
+  return !idles(F / 128.0, F / 128) && !idles(d / 256.0, (d + 255) / 256);
 }
 
 cudaError_t launch_ffn_pair_gate_up(const FfnArgs &a, cudaStream_t s) { return launch_phase<true>(a, s); }

@@ -1,8 +1,9 @@
 """The CTA-pair FFN kernels (many tokens per expert) against the oracle, on
 plain and packed weights (the same bits), at the edges of their tiles: token
-counts around 32 and 256, an odd number of 128-row blocks in d, one K step
-pair, experts with few tokens beside full ones, shared experts, and a rank of
-an expert-parallel layer."""
+counts around 32 and 256, an odd number of 128-row blocks in d, two K steps,
+experts with few tokens beside full ones, shared experts, few tokens per
+expert (batches of one, two and five 32-token chunks), repeated calls, and the
+ranks of an expert-parallel layer."""
 import pytest
 import torch
 
@@ -25,7 +26,8 @@ def _inputs(w, n_shared):
     (2, 2, 128, 128, 64, W.MODE_TOPK, 0), (4, 4, 384, 256, 255, W.MODE_TOPK, 0),
     (2, 2, 256, 384, 256, W.MODE_TOPK, 1), (3, 3, 640, 128, 257, W.MODE_TOPK, 0),
     (8, 2, 256, 256, 1000, W.MODE_TOPK, 2), (32, 4, 128, 384, 700, W.MODE_BATCH, 0),
-    (16, 3, 2048, 256, 513, W.MODE_HIER, 0)])
+    (16, 3, 2048, 256, 513, W.MODE_HIER, 0), (2, 2, 512, 128, 30, W.MODE_TOPK, 0),
+    (38, 8, 512, 256, 63, W.MODE_TOPK, 1), (38, 4, 512, 256, 150, W.MODE_TOPK, 0)])
 def test_pair_forward(X, N, k, d, F, B, mode, n_shared):  # noqa: F811
     w = W.TINY.with_(N=N, k=k, d=d, F=F, B=B, mode=mode, budget=6, k0=0, m_r=2,
                      tokens_per_request=3 if mode == W.MODE_HIER else 1, x_kind="domains")
@@ -35,6 +37,7 @@ def test_pair_forward(X, N, k, d, F, B, mode, n_shared):  # noqa: F811
     compare(w, g, x, W_g, weights, shared=shared)
     pk, ps = X.Packed(*weights), X.Packed(*shared) if shared else None
     y = run_one_gpu(X, w, x, W_g, pk, shared=ps)["y"]
+    assert torch.equal(y, run_one_gpu(X, w, x, W_g, pk, shared=ps)["y"])
     assert torch.equal(y.cpu().double(), torch.from_numpy(g["y"])), "packed and plain weights differ"
 
 
