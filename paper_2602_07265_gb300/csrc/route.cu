@@ -64,20 +64,21 @@ __device__ __forceinline__ float canonical_sum(const float *__restrict__ p, int 
 //
 // Up to 8 candidates per lane the lane keeps (key, index) pairs sorted best
 // first in registers (a bitonic network).  At 32 that is 64 registers and 240
-// exchanges, which spilled (10 KB of spill stores in score_kernel<32>): the
-// lane then keeps the keys alone, unsorted, and the winner scans them for its
-// next best (one lane, about 100 instructions a round).  Routing at N = 1000,
-// B = 100 on GB300 (whole call): 136 -> 35.6 us.
+// exchanges, which spilled (10 KB of spill stores in score_kernel<32>): from 16
+// on the lane keeps the keys alone, unsorted, and the winner scans them for its
+// next best (one lane, about 3 instructions a candidate).  Routing on GB300
+// (whole call): N = 1000, B = 100 136 -> 35.6 us; N = 512, B = 8192 with 16
+// candidates per lane instead of 32 122.7 -> 91.9 us, N = 400, B = 200 36.1 -> 28.3.
 constexpr int kSortedQ = 8;
 
-template <int Q>
-struct LaneList {   // Q <= kSortedQ
+template <int Q, bool kSorted = (Q <= kSortedQ)>
+struct LaneList {
   uint32_t key[Q];
   int idx[Q];
 };
-template <>
-struct LaneList<32> {
-  uint32_t key[32];   // slot q: candidate j0 + lane + 32 q; 0 once taken
+template <int Q>
+struct LaneList<Q, false> {
+  uint32_t key[Q];    // slot q: candidate j0 + lane + 32 q; 0 once taken
   int j0;
   uint32_t best;      // the lane's largest key and its (lowest) slot
   int bq;
@@ -1755,6 +1756,7 @@ cudaError_t launch_route(const RouteArgs &a, cudaStream_t s) {
   if (a.N <= 64) return launch_route_q<2>(a, s);
   if (a.N <= 128) return launch_route_q<4>(a, s);
   if (a.N <= 256) return launch_route_q<8>(a, s);
+  if (a.N <= 512) return launch_route_q<16>(a, s);
   return launch_route_q<32>(a, s);
 }
 

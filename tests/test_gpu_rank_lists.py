@@ -1,5 +1,6 @@
-"""Ranking with more than 256 experts (unsorted lane lists) against the oracle,
-bit for bit: ties, every mode, |S| on both sides of each compact list length."""
+"""Ranking with more than 256 experts (unsorted lane lists of 16 and 32) against
+the oracle, bit for bit: ties, every mode, both sides of 512 experts, |S| on
+both sides of each compact list length."""
 import pytest
 
 from paper_2602_07265_gb300 import workloads as W
@@ -9,7 +10,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("N,B,k,mode,budget,prm", [
-    (257, 33, 16, W.MODE_TOPK, 0, {}), (1024, 40, 16, W.MODE_TOPK, 0, {}),
+    (257, 33, 16, W.MODE_TOPK, 0, {}), (512, 40, 16, W.MODE_TOPK, 0, {}), (513, 40, 16, W.MODE_TOPK, 0, {}),
+    (512, 97, 8, W.MODE_BATCH, 257, dict(k0=1)), (384, 66, 8, W.MODE_HIER, 3, dict(k0=1, m_r=5, tokens_per_request=3)), (1024, 40, 16, W.MODE_TOPK, 0, {}),
     (512, 70, 8, W.MODE_BATCH, 64, dict(k0=0)), (512, 70, 8, W.MODE_BATCH, 65, dict(k0=0)),
     (700, 97, 8, W.MODE_BATCH, 128, dict(k0=0)), (700, 97, 8, W.MODE_BATCH, 256, dict(k0=0)),
     (1000, 97, 8, W.MODE_BATCH, 257, dict(k0=0)), (960, 66, 5, W.MODE_GROUP, 0, dict(k0=2, n_groups=4, m_g=40)),
