@@ -1367,6 +1367,16 @@ __global__ void __launch_bounds__(kRouteThreads, 1) topk_kernel(RouteArgs a) {
   }
 }
 
+// Clears the arrival counters of a routing call (no router kernel before it).
+// A kernel of the chain instead of a memset, which the next kernel's launch
+// would have to wait for (routing on GB300, N = 256: B = 256 26.2 -> 23.0 us,
+// N = 400, B = 200 29.4 -> 26.0 us).
+__global__ void clear_kernel(int32_t *done) {
+  pdl_wait();
+  pdl_trigger();
+  if (threadIdx.x < 4) done[threadIdx.x] = 0;
+}
+
 // Row of pair q = t * k + s: final in pos[q] for up to kFuseChunks chunks
 // (first == nullptr), else its rank plus the first row of (chunk, expert).
 __device__ __forceinline__ int pair_row(const int32_t *ids, const int32_t *pos, const int32_t *first,
@@ -1750,6 +1760,10 @@ cudaError_t launch_route_q(const RouteArgs &a, cudaStream_t s) {
   e = launch_pdl(refine_kernel<kQ>, dim3(C), dim3(kRouteThreads), 0, s, b);
   if (e != cudaSuccess || a.perm_out == nullptr) return e;
   return launch_scatter(a, s);
+}
+
+cudaError_t launch_clear(int32_t *done, cudaStream_t s) {
+  return launch_pdl(clear_kernel, dim3(1), dim3(32), 0, s, done);
 }
 
 cudaError_t launch_route(const RouteArgs &a, cudaStream_t s) {

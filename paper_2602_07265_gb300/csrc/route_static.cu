@@ -179,6 +179,6 @@ extern "C" int xshare_route_static(const float *scores, int B, int N, int k, int
   // The three arrival counters must start at zero; every other scratch word is
   // written before it is read.
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(a.done, 0, 3 * sizeof(int32_t), s) != cudaSuccess) return XS_ERR_CUDA;
+  if (launch_clear(a.done, s) != cudaSuccess) return XS_ERR_CUDA;
   return launch_route(a, s) == cudaSuccess ? XS_OK : XS_ERR_CUDA;
 }

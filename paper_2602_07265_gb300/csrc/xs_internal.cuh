@@ -186,6 +186,8 @@ struct RouteArgs {
 };
 
 cudaError_t launch_route(const RouteArgs &a, cudaStream_t s);
+// Clears the arrival counters done[0 .. 3] for a launch_route that follows.
+cudaError_t launch_clear(int32_t *done, cudaStream_t s);
 // Router logits for B < kRouterTcMinB.  d outside [kRouterSplitMinD,
 // kRouterSplitMaxD]: whole-d blocks of 8 tokens x 4 experts (route.cu),
 // h[t][e].  d inside: d-sliced blocks (router_split.cu), h[s][t][e] for s <
