@@ -132,7 +132,7 @@ Plan make_plan(int B, int N, int k, int d, int F, bool with_ffn, int n_sms, int 
     o = align_up(o + bytes);
     return r;
   };
-  const bool split = with_ffn && B < kRouterTcMinB && d >= kRouterSplitMinD && d <= kRouterSplitMaxD;
+  const bool split = with_ffn && !router_on_tensor_cores(B, N, d) && d >= kRouterSplitMinD && d <= kRouterSplitMaxD;
   const int h_splits = split ? router_split_count(B, N, d, n_sms) : 1;
   pl.h = take((size_t)h_splits * B * N * 4);
   pl.p = take((size_t)B * N * 4);
@@ -316,7 +316,7 @@ int xs::forward_impl(const FwdCall &c, FwdStep step) {
   cudaError_t re;
   int32_t *rstat = at<int32_t>(workspace, pl.rstat);
   a.router_status = rstat;
-  if (B >= kRouterTcMinB) {
+  if (router_on_tensor_cores(B, N, d)) {
     int grid = 0;
     re = launch_router_tc(c.x, c.W_g, h, B, N, d, a.done, rstat, sms, &grid, s);
     a.router_ctas = grid;
