@@ -145,8 +145,9 @@ __device__ __forceinline__ void lane_sort(LaneList<Q> &L) {
 }
 
 // Takes up to `count` candidates best first, calling emit(r, index, score)
-// on every lane; returns how many were taken.
-template <int Q, class Emit>
+// on every lane; returns how many were taken.  The list can be taken from
+// again only if kMore: otherwise the last winner is not replaced.
+template <int Q, bool kMore = false, class Emit>
 __device__ __forceinline__ int lane_take(LaneList<Q> &L, int count, Emit emit) {
   int r = 0;
   for (; r < count; ++r) {
@@ -164,7 +165,7 @@ __device__ __forceinline__ int lane_take(LaneList<Q> &L, int count, Emit emit) {
     const uint32_t cand = head == mx ? static_cast<uint32_t>(head_idx) : 0xffffffffu;
     const int win = static_cast<int>(__reduce_min_sync(kFull, cand));
     emit(r, win, key_score(mx));
-    if (head == mx && head_idx == win) {
+    if ((kMore || r + 1 < count) && head == mx && head_idx == win) {
       if constexpr (Q <= kSortedQ) {
 #pragma unroll
         for (int q = 0; q + 1 < Q; ++q) {
@@ -1186,7 +1187,7 @@ __global__ void __launch_bounds__(kRouteThreads, 1) score_kernel(RouteArgs a) {
       while (f < target) {
         float v = 0.f;
         int id = -1;
-        if (lane_take<kQ>(L, 1, [&](int, int e, float sv) {
+        if (lane_take<kQ, true>(L, 1, [&](int, int e, float sv) {
               id = e;
               v = sv;
             }) == 0)

@@ -48,3 +48,36 @@ def test_pair_expert_parallel(X):  # noqa: F811
     one = run_one_gpu(X, w, x, W_g, pk, shared=ps)["y"]
     y = run_ep(X, w, x, W_g, pk, 4, shared=ps)[0]
     assert torch.equal(y, one)   # no unit is cut: every row is the same bits on any rank
+
+
+def test_pair_graph_and_streams(X):  # noqa: F811
+    """A stack captured into a graph gives the direct call's bits; forwards on
+    two streams with workspaces of their own give the results they give alone."""
+    w = W.TINY.with_(N=8, k=2, d=256, F=256, B=600, mode=W.MODE_TOPK, x_kind="domains")
+    x, W_g, weights, _ = _inputs(w, 0)
+    dev = torch.device("cuda")
+    prm, pk, x, W_g = X.route_params(**w.params()), X.Packed(*weights), x.to(dev), W_g.to(dev)
+    size = X.xshare_workspace_size(w.B, w.N, w.k, w.d, w.F, w.mode, prm)
+    ws = [torch.empty(size, dtype=torch.uint8, device=dev) for _ in range(3)]
+    layers = [(W_g, pk)] * 3
+    h = [torch.empty(3, w.B, w.d, dtype=torch.bfloat16, device=dev) for _ in range(2)]
+    X.xshare_stack_forward(x, layers, w.k, 0, w.mode, prm, h[0], ws[0])
+    torch.cuda.synchronize()
+    g = X.StackGraph(x, layers, w.k, 0, w.mode, prm, h[1], ws[1])
+    for _ in range(3):
+        g.launch()
+    torch.cuda.synchronize()
+    assert torch.equal(h[0].view(torch.int16), h[1].view(torch.int16))
+    xs = [x, x.flip(0).contiguous()]
+    alone = [torch.empty_like(x) for _ in xs]
+    both = [torch.empty_like(x) for _ in xs]
+    for i, xi in enumerate(xs):
+        X.xshare_moe_forward_packed(xi, W_g, pk, w.k, 0, w.mode, prm, alone[i], ws[0])
+        torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in xs]
+    for _ in range(5):
+        for i, xi in enumerate(xs):
+            X.xshare_moe_forward_packed(xi, W_g, pk, w.k, 0, w.mode, prm, both[i], ws[1 + i], stream=streams[i])
+    torch.cuda.synchronize()
+    for a, b in zip(alone, both):
+        assert torch.equal(a.view(torch.int16), b.view(torch.int16))
