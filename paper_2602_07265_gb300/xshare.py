@@ -130,16 +130,24 @@ def xshare_strerror(code: int) -> str:
     return LIB.xshare_strerror(int(code)).decode()
 
 
-def _ptr(t: Optional[torch.Tensor], dtype, name: str, numel: Optional[int] = None) -> Optional[int]:
+def _device_of(t: torch.Tensor) -> int:
+    """The current device, looked up once per call (-1 without a CUDA tensor)."""
+    return torch.cuda.current_device() if t.is_cuda else -1
+
+
+def _ptr(t: Optional[torch.Tensor], dtype, name: str, numel: Optional[int] = None,
+         device: Optional[int] = None) -> Optional[int]:
+    """t's device pointer after the checks; `device`: the current device, if the
+    caller has looked it up."""
     if t is None:
         return None
     if not t.is_cuda:
         raise ValueError(f"{name} must be a CUDA tensor")
-    if t.device.index != torch.cuda.current_device():
+    if t.get_device() != (torch.cuda.current_device() if device is None else device):
         # The library launches on the current device.
         raise ValueError(f"{name} is on {t.device}, the current device is "
                          f"cuda:{torch.cuda.current_device()}")
-    if t.dtype != dtype:
+    if t.dtype is not dtype:
         raise ValueError(f"{name} must be {dtype}, got {t.dtype}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
@@ -173,14 +181,15 @@ def xshare_route(scores: torch.Tensor, k: int, budget: int, mode: int, params: R
                  perm: Optional[torch.Tensor] = None, stream=None) -> None:
     """Selection + refinement (+ permutation) on fp32 scores [B, N]; see xshare.h."""
     B, N = scores.shape
+    dev = _device_of(scores)
     rc = LIB.xshare_route(
-        _ptr(scores, torch.float32, "scores"), B, N, k, budget, mode, ctypes.byref(params),
-        _ptr(sel_mask, torch.uint8, "sel_mask", N), _ptr(topk_ids, torch.int32, "topk_ids", B * k),
-        _ptr(topk_w, torch.float32, "topk_w", B * k), _ptr(stats, torch.int32, "stats", STATS_WORDS),
-        _ptr(expert_counts, torch.int32, "expert_counts", N),
-        _ptr(expert_offsets, torch.int32, "expert_offsets", N + 1),
-        _ptr(perm, torch.int32, "perm", B * k),
-        _ptr(workspace, torch.uint8, "workspace"), workspace.numel(), _stream(stream))
+        _ptr(scores, torch.float32, "scores", None, dev), B, N, k, budget, mode, ctypes.byref(params),
+        _ptr(sel_mask, torch.uint8, "sel_mask", N, dev), _ptr(topk_ids, torch.int32, "topk_ids", B * k, dev),
+        _ptr(topk_w, torch.float32, "topk_w", B * k, dev), _ptr(stats, torch.int32, "stats", STATS_WORDS, dev),
+        _ptr(expert_counts, torch.int32, "expert_counts", N, dev),
+        _ptr(expert_offsets, torch.int32, "expert_offsets", N + 1, dev),
+        _ptr(perm, torch.int32, "perm", B * k, dev),
+        _ptr(workspace, torch.uint8, "workspace", None, dev), workspace.numel(), _stream(stream))
     _check(rc, "xshare_route")
 
 
@@ -196,13 +205,14 @@ def xshare_route_static(scores: torch.Tensor, k: int, budget: int, mode: int,
     """xshare_route without a workspace, for callers that may not allocate
     device memory (B <= STATIC_MAX_B; see xshare.h)."""
     B, N = scores.shape
+    dev = _device_of(scores)
     rc = LIB.xshare_route_static(
-        _ptr(scores, torch.float32, "scores"), B, N, k, budget, mode, ctypes.byref(params),
-        _ptr(sel_mask, torch.uint8, "sel_mask", N), _ptr(topk_ids, torch.int32, "topk_ids", B * k),
-        _ptr(topk_w, torch.float32, "topk_w", B * k), _ptr(stats, torch.int32, "stats", STATS_WORDS),
-        _ptr(expert_counts, torch.int32, "expert_counts", N),
-        _ptr(expert_offsets, torch.int32, "expert_offsets", N + 1),
-        _ptr(perm, torch.int32, "perm", B * k), _stream(stream))
+        _ptr(scores, torch.float32, "scores", None, dev), B, N, k, budget, mode, ctypes.byref(params),
+        _ptr(sel_mask, torch.uint8, "sel_mask", N, dev), _ptr(topk_ids, torch.int32, "topk_ids", B * k, dev),
+        _ptr(topk_w, torch.float32, "topk_w", B * k, dev), _ptr(stats, torch.int32, "stats", STATS_WORDS, dev),
+        _ptr(expert_counts, torch.int32, "expert_counts", N, dev),
+        _ptr(expert_offsets, torch.int32, "expert_offsets", N + 1, dev),
+        _ptr(perm, torch.int32, "perm", B * k, dev), _stream(stream))
     _check(rc, "xshare_route_static")
 
 
@@ -223,6 +233,7 @@ def xshare_moe_forward(x: torch.Tensor, W_g: torch.Tensor, W_gate: torch.Tensor,
     torch.cuda.Event objects) the profiled entry point records them between
     the kernel launches."""
     B, d = x.shape
+    dev = _device_of(x)
     N = W_g.shape[0]
     F = W_gate.shape[1]
     if W_g.shape[1] != d or tuple(W_gate.shape) != (N, F, d) or tuple(W_up.shape) != (N, F, d) \
@@ -236,19 +247,19 @@ def xshare_moe_forward(x: torch.Tensor, W_g: torch.Tensor, W_gate: torch.Tensor,
         if tuple(S_gate.shape) != (Ns, F, d) or tuple(S_up.shape) != (Ns, F, d) \
                 or tuple(S_down.shape) != (Ns, d, F):
             raise ValueError("inconsistent shared-expert shapes: [Ns,F,d], [Ns,F,d], [Ns,d,F]")
-        sh = SharedExperts(_ptr(S_gate, torch.bfloat16, "S_gate"),
-                           _ptr(S_up, torch.bfloat16, "S_up"),
-                           _ptr(S_down, torch.bfloat16, "S_down"), Ns)
+        sh = SharedExperts(_ptr(S_gate, torch.bfloat16, "S_gate", None, dev),
+                           _ptr(S_up, torch.bfloat16, "S_up", None, dev),
+                           _ptr(S_down, torch.bfloat16, "S_down", None, dev), Ns)
     args = [
-        _ptr(x, torch.bfloat16, "x"), _ptr(W_g, torch.float32, "W_g"),
-        _ptr(W_gate, torch.bfloat16, "W_gate"), _ptr(W_up, torch.bfloat16, "W_up"),
-        _ptr(W_down, torch.bfloat16, "W_down"), B, d, F, N, k, budget, mode,
+        _ptr(x, torch.bfloat16, "x", None, dev), _ptr(W_g, torch.float32, "W_g", None, dev),
+        _ptr(W_gate, torch.bfloat16, "W_gate", None, dev), _ptr(W_up, torch.bfloat16, "W_up", None, dev),
+        _ptr(W_down, torch.bfloat16, "W_down", None, dev), B, d, F, N, k, budget, mode,
         ctypes.byref(params), ctypes.byref(sh) if sh is not None else None,
-        _ptr(y, torch.bfloat16, "y"),
-        _ptr(scores_out, torch.float32, "scores_out", B * N),
-        _ptr(sel_mask, torch.uint8, "sel_mask", N), _ptr(topk_ids, torch.int32, "topk_ids", B * k),
-        _ptr(topk_w, torch.float32, "topk_w", B * k), _ptr(stats, torch.int32, "stats", STATS_WORDS),
-        _ptr(workspace, torch.uint8, "workspace"), workspace.numel(), _stream(stream)]
+        _ptr(y, torch.bfloat16, "y", None, dev),
+        _ptr(scores_out, torch.float32, "scores_out", B * N, dev),
+        _ptr(sel_mask, torch.uint8, "sel_mask", N, dev), _ptr(topk_ids, torch.int32, "topk_ids", B * k, dev),
+        _ptr(topk_w, torch.float32, "topk_w", B * k, dev), _ptr(stats, torch.int32, "stats", STATS_WORDS, dev),
+        _ptr(workspace, torch.uint8, "workspace", None, dev), workspace.numel(), _stream(stream)]
     if stage_events is None:
         _check(LIB.xshare_moe_forward(*args), "xshare_moe_forward")
         return
@@ -306,6 +317,7 @@ def xshare_moe_forward_packed(x: torch.Tensor, W_g: torch.Tensor, experts: Packe
                               stage_events: Optional[list] = None) -> None:
     """xshare_moe_forward on packed expert weights; see xshare.h."""
     B, d = x.shape
+    dev = _device_of(x)
     N = W_g.shape[0]
     if experts.n != N or experts.d != d or tuple(y.shape) != (B, d) or W_g.shape[1] != d:
         raise ValueError("inconsistent shapes")
@@ -321,13 +333,13 @@ def xshare_moe_forward_packed(x: torch.Tensor, W_g: torch.Tensor, experts: Packe
                 ev.record()
             handles[i] = ev.cuda_event
     rc = LIB.xshare_moe_forward_packed(
-        _ptr(x, torch.bfloat16, "x"), _ptr(W_g, torch.float32, "W_g"), ctypes.byref(ex), B, d,
+        _ptr(x, torch.bfloat16, "x", None, dev), _ptr(W_g, torch.float32, "W_g", None, dev), ctypes.byref(ex), B, d,
         experts.F, N, k, budget, mode, ctypes.byref(params),
-        ctypes.byref(sh) if sh is not None else None, _ptr(y, torch.bfloat16, "y"),
-        _ptr(scores_out, torch.float32, "scores_out", B * N),
-        _ptr(sel_mask, torch.uint8, "sel_mask", N), _ptr(topk_ids, torch.int32, "topk_ids", B * k),
-        _ptr(topk_w, torch.float32, "topk_w", B * k), _ptr(stats, torch.int32, "stats", STATS_WORDS),
-        _ptr(workspace, torch.uint8, "workspace"), workspace.numel(), _stream(stream), handles)
+        ctypes.byref(sh) if sh is not None else None, _ptr(y, torch.bfloat16, "y", None, dev),
+        _ptr(scores_out, torch.float32, "scores_out", B * N, dev),
+        _ptr(sel_mask, torch.uint8, "sel_mask", N, dev), _ptr(topk_ids, torch.int32, "topk_ids", B * k, dev),
+        _ptr(topk_w, torch.float32, "topk_w", B * k, dev), _ptr(stats, torch.int32, "stats", STATS_WORDS, dev),
+        _ptr(workspace, torch.uint8, "workspace", None, dev), workspace.numel(), _stream(stream), handles)
     _check(rc, "xshare_moe_forward_packed")
 
 
@@ -341,18 +353,19 @@ def xshare_moe_forward_ep(x: torch.Tensor, W_g: torch.Tensor, local_experts: Pac
     """This rank's part of an expert-parallel layer forward (routing of the
     whole batch, the FFN of expert group `rank`); see xshare.h."""
     B, d = x.shape
+    dev = _device_of(x)
     N = W_g.shape[0]
     if local_experts.n * n_ranks != N or local_experts.d != d or W_g.shape[1] != d:
         raise ValueError("inconsistent shapes")
     ex = local_experts.struct()
     sh = shared.struct() if shared is not None else None
     rc = LIB.xshare_moe_forward_ep(
-        _ptr(x, torch.bfloat16, "x"), _ptr(W_g, torch.float32, "W_g"), ctypes.byref(ex), B, d,
+        _ptr(x, torch.bfloat16, "x", None, dev), _ptr(W_g, torch.float32, "W_g", None, dev), ctypes.byref(ex), B, d,
         local_experts.F, N, k, budget, mode, ctypes.byref(params),
         ctypes.byref(sh) if sh is not None else None, n_ranks, rank,
-        _ptr(sel_mask, torch.uint8, "sel_mask", N), _ptr(topk_ids, torch.int32, "topk_ids", B * k),
-        _ptr(topk_w, torch.float32, "topk_w", B * k), _ptr(stats, torch.int32, "stats", STATS_WORDS),
-        _ptr(workspace, torch.uint8, "workspace"), workspace.numel(), _stream(stream))
+        _ptr(sel_mask, torch.uint8, "sel_mask", N, dev), _ptr(topk_ids, torch.int32, "topk_ids", B * k, dev),
+        _ptr(topk_w, torch.float32, "topk_w", B * k, dev), _ptr(stats, torch.int32, "stats", STATS_WORDS, dev),
+        _ptr(workspace, torch.uint8, "workspace", None, dev), workspace.numel(), _stream(stream))
     _check(rc, "xshare_moe_forward_ep")
 
 
