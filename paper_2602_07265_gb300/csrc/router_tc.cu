@@ -288,20 +288,40 @@ __global__ void __launch_bounds__(kThreads, 1) router_tc_kernel(const __grid_con
 
   // Rows [split * 128 / S, (split + 1) * 128 / S) of the tile, summed over
   // the S partials in rank order.
+  // Four experts per thread and step: one at a time a CTA of a small cluster
+  // went round the loop 9 (S = 2) or 18 times (S = 1), a remote load's latency
+  // each (router 46.4 -> 40.3 us at N = 128, d = 2048, B = 6000, where S = 1;
+  // 32 -> 30 us at N = 64, B = 8192, where S = 2; equal for S >= 4).
   const int rows = kBM / S, r_begin = split * rows;
-  for (int e = threadIdx.x; e < rows * kNt; e += kThreads) {
-    const int r = r_begin + e / kNt, c = e % kNt;
+  for (int e = threadIdx.x; e < rows * (kNt / 4); e += kThreads) {
+    const int r = r_begin + e / (kNt / 4), c = e % (kNt / 4) * 4;
     const int t = m0 + r, j = n0 + c;
     const uint32_t a = sbase + static_cast<uint32_t>((r * (kNt + 4) + c) * 4);
-    float part[16];  // all remote loads in flight first, then the sum in rank order
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s0 = 0; s0 < S; s0 += 8) {
+      float4 part[8];  // the loads in flight first, then the sum in rank order
 #pragma unroll
-    for (int src = 0; src < 16; ++src)
-      part[src] = src < S ? ld_cluster_f32(a, static_cast<uint32_t>(src)) : 0.f;
-    float v = 0.f;
+      for (int i = 0; i < 8; ++i)
+        part[i] = s0 + i < S ? ld_cluster_f32x4(a, static_cast<uint32_t>(s0 + i)) : v;
 #pragma unroll
-    for (int src = 0; src < 16; ++src)
-      if (src < S) v = __fadd_rn(v, part[src]);
-    if (t < p.B && j < p.N) p.h[static_cast<size_t>(t) * p.N + j] = v;
+      for (int i = 0; i < 8; ++i)
+        if (s0 + i < S) {
+          v.x = __fadd_rn(v.x, part[i].x);
+          v.y = __fadd_rn(v.y, part[i].y);
+          v.z = __fadd_rn(v.z, part[i].z);
+          v.w = __fadd_rn(v.w, part[i].w);
+        }
+    }
+    if (t >= p.B) continue;
+    float *dst = p.h + static_cast<size_t>(t) * p.N + j;
+    if (p.N % 4 == 0) {  // j is a multiple of 4: all four or none
+      if (j < p.N) *reinterpret_cast<float4 *>(dst) = v;
+    } else {
+      if (j < p.N) dst[0] = v.x;
+      if (j + 1 < p.N) dst[1] = v.y;
+      if (j + 2 < p.N) dst[2] = v.z;
+      if (j + 3 < p.N) dst[3] = v.w;
+    }
   }
   cluster_sync();  // no CTA leaves while another still reads its shared memory
   if (threadIdx.x == 0) p.status[blockIdx.x] = *abort_flag ? XS_DEV_TIMEOUT : XS_DEV_OK;

@@ -247,13 +247,16 @@ __device__ __forceinline__ void cluster_sync() {
                    "memory");
 }
 
-// fp32 load from the shared memory of CTA `rank` of the cluster, at the
-// offset that `saddr` has in this CTA's shared memory.
-__device__ __forceinline__ float ld_cluster_f32(uint32_t saddr, uint32_t rank) {
+// Four fp32 values from the shared memory of CTA `rank` of the cluster, at the
+// (16-byte aligned) offset that `saddr` has in this CTA's shared memory.
+__device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t saddr, uint32_t rank) {
   uint32_t remote;
-  float v;
+  float4 v;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(saddr), "r"(rank));
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(remote) : "memory");
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(remote)
+               : "memory");
   return v;
 }
 

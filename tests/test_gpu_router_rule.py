@@ -12,7 +12,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("N,d,B", [
     (64, 2048, 63), (64, 2048, 64), (64, 2048, 256), (64, 2048, 257), (100, 512, 655), (100, 512, 656),
-    (8, 3968, 1057), (8, 3968, 1058), (9, 4096, 64), (1024, 128, 256), (1024, 128, 257)])
+    (8, 3968, 1057), (8, 3968, 1058), (9, 4096, 64), (1024, 128, 256), (1024, 128, 257),
+    (66, 512, 3000), (130, 512, 8191), (132, 512, 8191)])
 def test_both_routers(X, N, d, B):  # noqa: F811
     w = W.TINY.with_(N=N, d=d, F=128, B=B, k=4, budget=6)
     x, W_g = W.router_inputs(w, seed=9)
