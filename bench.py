@@ -326,6 +326,14 @@ def algorithmic_bytes(w: W.Workload, n_used: int, n_pairs: int, n_shared: int = 
     }
 
 
+def layer_launches(w: W.Workload) -> int:
+    """Kernels of one layer forward: router, selection, refinement (part of the
+    selection kernel for up to two 32-token chunks and for TOPK), gather,
+    gate/up, down, combine."""
+    from paper_2602_07265_gb300 import xshare as X
+    return X.N_STAGES - (1 if w.B <= 64 or w.mode == W.MODE_TOPK else 0)
+
+
 def run_gpu(args, w: W.Workload, rank: int, world: int, local: int) -> dict:
     from paper_2602_07265_gb300 import _build
     _build.build()
@@ -479,9 +487,7 @@ def run_gpu(args, w: W.Workload, rank: int, world: int, local: int) -> dict:
     barrier(world)
     e2e_ms = reduce_max(e0.elapsed_time(e1), world, dev)
 
-    # router, selection, [refinement: its own kernel beyond two 32-token
-    # chunks], gather, gate/up, down, combine
-    launches_per_step = X.N_STAGES - (1 if (w.B + 31) // 32 <= 2 else 0)
+    launches_per_step = layer_launches(w)
     out = {
         "metric": METRIC,
         "value": tokens_total / (ms_total * 1e-3),
@@ -626,7 +632,7 @@ def run_gpu_ep(args, w: W.Workload, rank: int, world: int, local: int) -> dict:
     torch.cuda.synchronize()
     barrier(world)
     e2e_ms = reduce_max(e0.elapsed_time(e1), world, dev)
-    launches = 7 - (1 if (w.B + 31) // 32 <= 2 else 0)
+    launches = layer_launches(w)
     return {
         "metric": METRIC, "value": w.B * K / (ms_total * 1e-3), "unit": "tokens/s",
         "n_gpus": world, "steps": K, "warmup": Wm, "ms_per_step": ms_total / K,
@@ -823,7 +829,7 @@ def run_gpu_stack(args, w: W.Workload, rank: int, world: int, local: int) -> dic
     barrier(world)
     e2e_ms = reduce_max(e0.elapsed_time(e1), world, dev)
     g.close()
-    launches_per_layer = X.N_STAGES - (1 if (w.B + 31) // 32 <= 2 else 0)
+    launches_per_layer = layer_launches(w)
     achieved = stack_bytes / step_s / 1e9
     return {
         "metric": METRIC,

@@ -248,8 +248,8 @@ int xshare_route_static(const float *scores, int B, int N, int k, int budget, in
 
 /* Kernel stages of xshare_moe_forward, in launch order: router logits,
  * selection (softmax, ranking, column scores, Algorithms 2-6), refinement
- * and permutation (inside the selection kernel for B <= 64, so its events
- * then enclose no kernel), token gather, SwiGLU gate/up, SwiGLU down,
+ * and permutation (inside the selection kernel for B <= 64 and for TOPK, so
+ * its events then enclose no kernel), token gather, SwiGLU gate/up, SwiGLU down,
  * weighted combine. */
 #define XS_N_STAGES 7
 

@@ -16,13 +16,14 @@
 //   - two 256-column TMEM accumulators let the epilogue of a unit run under
 //     the MMAs of the next.
 // Measured on GB300 (whole layer, ffn_tc.cu -> this): d = 2048, F = 1024, 48
-// experts, B = 8192 (1365 tokens an expert) 1479 -> 735 us (gate/up 829 -> 340
-// us, 1.6 PFLOP/s; down 436 -> 212 us, which also writes 537 MB of fp32 rows);
-// d = 2048, F = 768, 128 experts, B = 2048 (128 tokens) 416 -> 310 us.  Four
+// experts, B = 8192 (1365 tokens an expert) 1479 -> 725 us (gate/up 829 -> 335
+// us, 1.64 PFLOP/s; down 436 -> 213 us, which also writes 537 MB of fp32 rows:
+// 178 us without the stores); d = 2048, F = 768, 128 experts, B = 2048 (128
+// tokens) 416 -> 284 us (gate/up 142 us for 805 MB of weights).  Four
 // pipeline stages instead of six cost 5 %, tiles dealt expert by expert to all
 // pairs (one row block at a time) 19 %.  With the loads left out the MMAs and
 // the epilogue of the first case's gate/up phase take 254 us (2.2 PFLOP/s), of
-// the second's 68 us (155 us with the loads, which stream 805 MB).
+// the second's 68 us.
 //
 // Unit: (tile of up to 256 tokens of one expert, block of weight rows).  The
 // weights are the MMA's M = 256 rows, 128 in each CTA; the tokens are its N
@@ -33,10 +34,11 @@
 // No unit is cut, so there are no partial sums and the result does not depend
 // on the schedule.
 //
-// Roles inside a CTA (64 + 32 kEpiWarps threads): warp 0 lane 0 loads this CTA's half of both
-// operands by TMA; in rank 0, warp 1 lane 0 issues the pair's MMAs; the other
-// warps (several per TMEM lane quarter, taking turns at 32 columns) drain this CTA's
-// accumulator.  Every mbarrier wait is bounded in time.
+// Roles inside a CTA (64 + 32 kEpiWarps threads): an elected lane of warp 0
+// loads this CTA's half of both operands by TMA; in rank 0, one of warp 1
+// issues the pair's MMAs; the other warps (two per TMEM lane quarter, taking
+// turns at 32 columns) drain this CTA's accumulator.  Every mbarrier wait is
+// bounded in time.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>

@@ -19,8 +19,8 @@
 // K order (deterministic) and runs the epilogue.  No CTA ever waits for
 // another.
 //
-// Roles inside a CTA (192 threads): warp 0 lane 0 issues TMA loads into a
-// ring of shared-memory stages; warp 1 lane 0 issues the MMAs into one of two
+// Roles inside a CTA (192 threads): an elected lane of warp 0 issues TMA loads
+// into a ring of shared-memory stages; one of warp 1 the MMAs into one of two
 // TMEM accumulator buffers; warps 2-5 (one TMEM lane quarter each) drain the
 // accumulators.  Every mbarrier wait is bounded in time.
 #include <cuda.h>

@@ -402,6 +402,9 @@ __device__ __forceinline__ void block_scan3(int (&v)[3], int (&tot)[3], int *s_t
 //       last takes the prefix sums over chunks and experts and writes the
 //       FFN tiles; the pairs are placed by the kernel after it.
 //
+// Up to kFuseChunks chunks score_kernel refines and permutes too; beyond them
+// topk_kernel does both kernels' work for TOPK, where S = E.
+//
 // "Last to finish" uses an arrival counter per group of CTAs (done[0] the
 // selection, done[1] the refinement, done[2] the union), cleared before the
 // first kernel of the call: every CTA writes its results, fences, and bumps

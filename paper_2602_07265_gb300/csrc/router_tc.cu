@@ -12,7 +12,7 @@
 //
 // Tiling: the MMA's M = 128 rows are tokens (A = x, K-major, 128-byte
 // swizzle, loaded by TMA), N = nt experts (B = the three weight planes,
-// written by four converter warps in the same swizzled layout), K = 16 per
+// written by the converter warps in the same swizzled layout), K = 16 per
 // instruction, 64 per pipeline stage.  An output tile of 128 tokens x nt
 // experts is computed by a cluster of S <= 16 CTAs, each over 1/S of d; the CTAs
 // park their fp32 partial tiles in shared memory and every CTA then adds up
@@ -27,7 +27,7 @@
 // round-to-nearest addition per stage, while the next stages are
 // multiplied into up to seven other TMEM buffers.
 //
-// Roles (448 threads): warp 0 lane 0 issues TMA, warp 1 lane 0 issues the
+// Roles (448 threads): an elected lane of warp 0 issues TMA, one of warp 1 the
 // MMAs, warps 2-5 and 6-9 convert the weight planes of the even and the odd
 // K steps (the conversion of a step is a chain of shared-memory round trips
 // and a proxy fence; with one group the router took 29.8 us between its events
