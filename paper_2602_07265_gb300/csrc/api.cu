@@ -367,7 +367,7 @@ int xs::forward_impl(const FwdCall &c, FwdStep step) {
       return XS_ERR_CUDA;
     return XS_OK;
   }
-  if (launch_combine(f.out, a.pos, a.w, a.meta, c.resid, c.y, B, d, k, n_shared, s) !=
+  if (launch_combine(f.out, f.act, a.pos, a.w, a.meta, c.resid, c.y, B, d, F, k, n_shared, s) !=
           cudaSuccess ||
       !mark(7))
     return XS_ERR_CUDA;
@@ -549,9 +549,9 @@ extern "C" int xshare_ep_combine(void *workspace, int B, int N, int k, int d, in
   const int rc = ep_plan(workspace, B, N, k, d, F, mode, prm, n_shared, &pl);
   if (rc != XS_OK) return rc;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  return launch_combine(at<float>(workspace, pl.out), at<int32_t>(workspace, pl.pos),
+  return launch_combine(at<float>(workspace, pl.out), nullptr, at<int32_t>(workspace, pl.pos),
                         at<float>(workspace, pl.w), at<Meta>(workspace, pl.meta), nullptr, y, B, d,
-                        k, n_shared, s) == cudaSuccess
+                        F, k, n_shared, s) == cudaSuccess
              ? XS_OK
              : XS_ERR_CUDA;
 }

@@ -1734,16 +1734,34 @@ __global__ void __launch_bounds__(256) gather_kernel(const uint16_t *__restrict_
     }
 }
 
+// Drops the 128-byte line at p (aligned) from L2 without writing it back.
+__device__ __forceinline__ void discard_line(const void *p) {
+  asm volatile("discard.global.L2 [%0], 128;" ::"l"(p) : "memory");
+}
+
 // ---- a9: y_t = [x_t +] sum over slots s < k' of w_ts * out[pos(t, s)]
 //              + sum over shared experts j of out[n_pairs + j * B + t], fp32, bf16 once.
 // The residual x_t is added first when `resid` is given (layer stacks).
-__global__ void __launch_bounds__(256) combine_kernel(const float *__restrict__ out,
+//
+// This is the last reader of the expert outputs and the activations.  Their
+// lines are still dirty in L2 and would be written back to HBM while the next
+// kernels stream weights.  With kLast the outputs are read with evict-first
+// priority, and the lines of a pair's output and activation row are discarded
+// (dropped without a write-back) once the warp has its values; reading them
+// again gives undefined data until they are written again.  Layer forward on
+// GB300, without -> with, us: plain top-k, d = 2048: N = 64, B = 512 154.6 ->
+// 151.4, 1024 178 -> 174.5, 2048 255 -> 247, 8192 715 -> 708; N = 128, B = 256
+// 208 -> 205, B = 2048 285 -> 277; N = 256, d = 7168, groups, B = 256 763 -> 754.
+// Discarding the gathered tokens as well (dead since gate/up) was slower by 1 to
+// 2 us; batching the loads of eight rows changed nothing.
+template <bool kLast>
+__global__ void __launch_bounds__(256) combine_kernel(const float *out, const uint16_t *act,
                                                       const int32_t *__restrict__ pos,
                                                       const float *__restrict__ w,
                                                       const Meta *__restrict__ meta,
                                                       const uint16_t *__restrict__ resid,
                                                       uint16_t *__restrict__ y, int B, int d,
-                                                      int k, int n_shared) {
+                                                      int F, int k, int n_shared) {
   __shared__ int32_t s_row[kMaxK];
   __shared__ float s_w[kMaxK];
   __shared__ int32_t s_kp, s_pairs;
@@ -1773,13 +1791,14 @@ __global__ void __launch_bounds__(256) combine_kernel(const float *__restrict__ 
   __syncthreads();
   pdl_wait();
   pdl_trigger();
-  if (c4 >= d / 4) return;
+  if (c4 >= d / 4) return;  // whole warps: d is a multiple of 128
   const int kp = s_kp;
+  auto load = [](const float4 *src) { return kLast ? __ldcs(src) : __ldg(src); };
   for (int s = 0; s < kp; ++s) {
     const int r = s_row[s];
     if (r < 0) continue;  // only with non-finite scores
     const float ws = s_w[s];
-    const float4 o = reinterpret_cast<const float4 *>(out + (size_t)r * d)[c4];
+    const float4 o = load(reinterpret_cast<const float4 *>(out + (size_t)r * d) + c4);
     acc.x = fmaf(ws, o.x, acc.x);
     acc.y = fmaf(ws, o.y, acc.y);
     acc.z = fmaf(ws, o.z, acc.z);
@@ -1787,7 +1806,7 @@ __global__ void __launch_bounds__(256) combine_kernel(const float *__restrict__ 
   }
   for (int j = 0; j < n_shared; ++j) {
     const size_t r = (size_t)s_pairs + (size_t)j * B + t;
-    const float4 o = reinterpret_cast<const float4 *>(out + r * d)[c4];
+    const float4 o = load(reinterpret_cast<const float4 *>(out + r * d) + c4);
     acc.x += o.x;
     acc.y += o.y;
     acc.z += o.z;
@@ -1799,6 +1818,19 @@ __global__ void __launch_bounds__(256) combine_kernel(const float *__restrict__ 
   v.x = *reinterpret_cast<uint32_t *>(&lo);
   v.y = *reinterpret_cast<uint32_t *>(&hi);
   reinterpret_cast<uint2 *>(y + (size_t)t * d)[c4] = v;
+  if (kLast) {
+    __syncwarp();  // every lane has used its values
+    // A warp has 128 columns: four lines of every output row, and its share of
+    // the activation row's lines.
+    const int lane = threadIdx.x & 31, part = lane & 3, warp = c4 >> 5, warps = d / 128;
+    for (int i = lane >> 2; i < kp + n_shared; i += 8) {
+      const int r = i < kp ? s_row[i] : s_pairs + (i - kp) * B + t;
+      if (r < 0) continue;
+      discard_line(out + static_cast<size_t>(r) * d + warp * 128 + part * 32);
+      for (int l = warp + part * warps; l < F / 64; l += 4 * warps)
+        discard_line(act + static_cast<size_t>(r) * F + l * 64);
+    }
+  }
 }
 
 }  // namespace
@@ -1876,12 +1908,13 @@ cudaError_t launch_gather(const uint16_t *x, const RouteArgs &a, uint16_t *xp, f
                     xp, zero_out, a.B, a.N, d, a.k, a.n_shared, per_block, pf);
 }
 
-cudaError_t launch_combine(const float *out, const int32_t *pos, const float *w,
-                           const Meta *meta, const uint16_t *resid, uint16_t *y, int B, int d,
+cudaError_t launch_combine(const float *out, const uint16_t *act, const int32_t *pos, const float *w,
+                           const Meta *meta, const uint16_t *resid, uint16_t *y, int B, int d, int F,
                            int k, int n_shared, cudaStream_t s) {
   dim3 grid((d / 4 + 255) / 256, B);
-  return launch_pdl(combine_kernel, grid, dim3(256), 0, s, out, pos, w, meta, resid, y, B, d, k,
-                    n_shared);
+  const bool last = act != nullptr && static_cast<long long>(B) * (k + n_shared) * d * 4 >= kDiscardBytes;
+  return launch_pdl(last ? combine_kernel<true> : combine_kernel<false>, grid, dim3(256), 0, s, out, act, pos,
+                    w, meta, resid, y, B, d, F, k, n_shared);
 }
 
 }  // namespace xs

@@ -53,6 +53,12 @@ constexpr int kChunk = 32;                   // tokens per selection CTA (= the 
 constexpr int kScoreRowBytes = 190 * 1024;   // score rows of a selection CTA at most
 constexpr int kFuseChunks = 2;               // up to this many chunks the selection CTA also refines
 constexpr int kMaxShared = 8;                // shared experts
+// The combine discards the layer's dead lines from this many bytes of expert
+// outputs on.  Without -> with, us: 4 MB (d = 2048, B = 64) plain top-k N = 64
+// 138.5 -> 138.1, N = 128 191.4 -> 190.3, 24 experts 69.0 -> 69.2; 6 MB (B = 96)
+// 140.1 -> 138.6, 196.1 -> 194.2, 32 experts 94.4 -> 94.8; 7 MB (d = 7168, B = 32)
+// 555.0 -> 552.5; 11 MB (B = 48) 661.3 -> 656.2; 2 MB: equal.
+constexpr long long kDiscardBytes = 6ll << 20;
 constexpr int kGatherPrefetchBytes = 256 * 1024;  // L2 warm-up per gate/up CTA (packed weights)
 // The same for the CTA-pair kernel, in total: layer forward at N = 64, d = 2048,
 // F = 1024, B = 512 without, 32, 64 and 96 MB 170.4, 168.3, 166.4, 166.9 us; no
@@ -223,8 +229,10 @@ int router_tc_ctas(int B, int N, int d, int n_sms);
 cudaError_t launch_router_tc(const uint16_t *x, const float *Wg, float *h, int B, int N, int d,
                              int32_t *done, int32_t *status, int n_sms, int *grid_out,
                              cudaStream_t s);
-cudaError_t launch_combine(const float *out, const int32_t *pos, const float *w,
-                           const Meta *meta, const uint16_t *resid, uint16_t *y, int B, int d,
+// act: the activations if nothing reads them or `out` afterwards (they may then
+// be discarded), else nullptr.
+cudaError_t launch_combine(const float *out, const uint16_t *act, const int32_t *pos, const float *w,
+                           const Meta *meta, const uint16_t *resid, uint16_t *y, int B, int d, int F,
                            int k, int n_shared, cudaStream_t s);
 // What the gather kernel needs to warm L2 with the gate/up kernel's first
 // weights (packed weights only; pk == nullptr: no warm-up).
