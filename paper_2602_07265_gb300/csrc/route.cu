@@ -1793,7 +1793,8 @@ __global__ void __launch_bounds__(256) combine_kernel(const float *out, const ui
   pdl_trigger();
   if (c4 >= d / 4) return;  // whole warps: d is a multiple of 128
   const int kp = s_kp;
-  auto load = [](const float4 *src) { return kLast ? __ldcs(src) : __ldg(src); };
+  // (__ldg in the second form cost 0.4 us at N = 64, d = 2048, B = 32.)
+  auto load = [](const float4 *src) { return kLast ? __ldcs(src) : *src; };
   for (int s = 0; s < kp; ++s) {
     const int r = s_row[s];
     if (r < 0) continue;  // only with non-finite scores
