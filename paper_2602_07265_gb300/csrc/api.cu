@@ -291,6 +291,8 @@ int xs::forward_impl(const FwdCall &c, FwdStep step) {
     f.S_down = shared->W_down;
   }
   f.n_shared = n_shared;
+  const long long xp_bytes = static_cast<long long>(B) * (k + n_shared) * d * 2;
+  f.drop_xp = xp_bytes >= kDropTokensMin && xp_bytes <= kDropTokensMax;
   f.xp = at<uint16_t>(workspace, pl.xp);
   f.act = at<uint16_t>(workspace, pl.act);
   f.out = at<float>(workspace, pl.out);

@@ -76,6 +76,7 @@ struct PairParams {
   xs_stats *stats;
   uint16_t *act_out;    // gate/up output [max_rows, M]
   float *out;           // down output [max_rows, M]
+  const uint16_t *drop; // down: nullable, the token rows [max_rows, M] that gate/up read
   int M;                // weight rows per expert: F (gate/up) or d (down)
   int K;                // reduction length: d (gate/up) or F (down)
   int n_routed;         // N: tiles of experts >= N use tmS
@@ -323,6 +324,13 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_pair_kernel(const __grid_cons
       if (elect_one()) mma_commit_pair_local(drain_bar);
       volatile int no_abort = 0;
       mbar_wait(drain_bar, 0, kWaitNs, &no_abort);
+    } else if (!kGateUp && p.drop != nullptr) {
+      // The rows of all tiles, in equal shares over the pairs that have work.
+      const Unit a = unit_at(0, false), b = unit_at(n_units - 1, false);
+      const int lines = (b.row0 + b.ntok - a.row0) * (p.M / 64);
+      const uint16_t *base = p.drop + static_cast<size_t>(a.row0) * p.M;
+      const int step = 32 * (n_pairs < n_units ? n_pairs : n_units);
+      for (int l = 32 * pair + lane; l < lines; l += step) discard_line(base + static_cast<size_t>(l) * 64);
     }
   } else {
     // ------------------------------------------------ epilogue
@@ -490,6 +498,7 @@ cudaError_t launch_phase(const FfnArgs &a, cudaStream_t s) {
   p.stats = a.stats;
   p.act_out = a.act;
   p.out = a.out;
+  p.drop = !kGateUp && a.drop_xp ? a.xp : nullptr;
   p.n_routed = a.N;
   p.expert_base = a.expert_base;
   cudaError_t e = cudaFuncSetAttribute(kernel_ptr<kGateUp>(), cudaFuncAttributeMaxDynamicSharedMemorySize,

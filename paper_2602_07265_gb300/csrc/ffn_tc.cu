@@ -78,6 +78,7 @@ struct TcParams {
   int32_t *cnt;         // [units] arrival counters, zeroed by the routing kernel
   uint16_t *act_out;    // gate/up output [max_rows, M]
   float *out;           // down output [max_rows, M]
+  const uint16_t *drop; // down: nullable, the token rows [max_rows, M] that gate/up read
   int M;                // weight rows per expert: F (gate/up) or d (down)
   int K;                // reduction length: d (gate/up) or F (down)
   int grid;
@@ -418,6 +419,13 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_tc_kernel(const __grid_consta
     const int q = warp & 3;                  // TMEM lane quarter of this warp
     const int row = q * 32 + lane;           // weight row inside the unit
     const bool leader = threadIdx.x == 64;
+    if (!kGateUp && p.drop != nullptr) {  // the rows of all tiles, in equal shares
+      const Tile a = p.tiles[wt.tile(0)], b = p.tiles[wt.tile(n_tiles - 1)];
+      const int lines = (b.row0 + b.ntok - a.row0) * (p.M / 64);
+      const uint16_t *base = p.drop + static_cast<size_t>(a.row0) * p.M;
+      for (int l = kEpiThreads * cta + static_cast<int>(threadIdx.x) - 64; l < lines; l += kEpiThreads * rg.G)
+        discard_line(base + static_cast<size_t>(l) * 64);
+    }
     for (int segi = 0; segi < n_seg; ++segi) {
       const Seg g = seg_at(segi);
       const long long u = g.u;
@@ -658,6 +666,7 @@ cudaError_t launch_ffn_down(const FfnArgs &a, cudaStream_t s) {
   p.part = static_cast<float *>(a.part);
   p.cnt = a.cnt + static_cast<size_t>(a.max_tiles) * (a.F / kBM);
   p.out = a.out;
+  p.drop = a.drop_xp ? a.xp : nullptr;
   p.M = a.d;
   p.K = a.F;
   p.grid = a.n_sms;

@@ -1734,11 +1734,6 @@ __global__ void __launch_bounds__(256) gather_kernel(const uint16_t *__restrict_
     }
 }
 
-// Drops the 128-byte line at p (aligned) from L2 without writing it back.
-__device__ __forceinline__ void discard_line(const void *p) {
-  asm volatile("discard.global.L2 [%0], 128;" ::"l"(p) : "memory");
-}
-
 // ---- a9: y_t = [x_t +] sum over slots s < k' of w_ts * out[pos(t, s)]
 //              + sum over shared experts j of out[n_pairs + j * B + t], fp32, bf16 once.
 // The residual x_t is added first when `resid` is given (layer stacks).
@@ -1752,8 +1747,8 @@ __device__ __forceinline__ void discard_line(const void *p) {
 // GB300, without -> with, us: plain top-k, d = 2048: N = 64, B = 512 154.6 ->
 // 151.4, 1024 178 -> 174.5, 2048 255 -> 247, 8192 715 -> 708; N = 128, B = 256
 // 208 -> 205, B = 2048 285 -> 277; N = 256, d = 7168, groups, B = 256 763 -> 754.
-// Discarding the gathered tokens as well (dead since gate/up) was slower by 1 to
-// 2 us; batching the loads of eight rows changed nothing.
+// Discarding the gathered tokens here as well was slower by 1 to 2 us (the down
+// kernel does it, for some sizes); batching the loads of eight rows changed nothing.
 template <bool kLast>
 __global__ void __launch_bounds__(256) combine_kernel(const float *out, const uint16_t *act,
                                                       const int32_t *__restrict__ pos,

@@ -43,6 +43,11 @@ cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, size_t 
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
+// Drops the 128-byte line at p (aligned) from L2 without writing it back.
+__device__ __forceinline__ void discard_line(const void *p) {
+  asm volatile("discard.global.L2 [%0], 128;" ::"l"(p) : "memory");
+}
+
 constexpr int kMaxN = 1024;     // experts
 constexpr int kMaxK = 16;       // top-k and warm-up k0
 constexpr int kMaxB = 8192;     // tokens
@@ -59,6 +64,14 @@ constexpr int kMaxShared = 8;                // shared experts
 // 140.1 -> 138.6, 196.1 -> 194.2, 32 experts 94.4 -> 94.8; 7 MB (d = 7168, B = 32)
 // 555.0 -> 552.5; 11 MB (B = 48) 661.3 -> 656.2; 2 MB: equal.
 constexpr long long kDiscardBytes = 6ll << 20;
+// The down kernel discards the gathered tokens, which only gate/up reads, if
+// they take this many bytes: fewer are gathered again before they are written
+// back, more have left L2 already.  Layer forward without -> with, us: 15 MB
+// (d = 7168, B = 128) 926.0 -> 928.0; 17 MB (d = 2048, B = 512) equal; 20 MB
+// 154.5 -> 154.1; 25 MB 161.6 -> 158.9; 29 MB (d = 7168, B = 256) 1113.7 -> 1103.9,
+// groups 756.6 -> 749.8; 43 MB 183.5 -> 180.7; 52 MB 199.3 -> 198.2; 67 MB equal;
+// 197 MB (B = 6000) 517.0 -> 521.4.
+constexpr long long kDropTokensMin = 16ll << 20, kDropTokensMax = 64ll << 20;
 constexpr int kGatherPrefetchBytes = 256 * 1024;  // L2 warm-up per gate/up CTA (packed weights)
 // The same for the CTA-pair kernel, in total: layer forward at N = 64, d = 2048,
 // F = 1024, B = 512 without, 32, 64 and 96 MB 170.4, 168.3, 166.4, 166.9 us; no
@@ -265,6 +278,7 @@ struct FfnArgs {
   const Tile *tiles;
   Meta *meta;
   xs_stats *stats;       // nullable
+  bool drop_xp;          // the down kernel discards the token rows (kDropTokensMin)
   void *part;            // partial-sum scratch
   int32_t *cnt;          // arrival counters (cleared by the routing kernel)
   int N, d, F, max_rows, max_tiles, n_sms;

@@ -1,6 +1,8 @@
-"""The combine that discards the layer's dead lines: sizes on both sides of its
-line (6 MB of expert outputs), more rows a token than a warp takes at once,
-rows of activations shorter and longer than the warps' shares, shared experts."""
+"""The kernels that discard dead lines.  The combine (outputs, activations):
+sizes on both sides of its line (6 MB of expert outputs), more rows a token than
+a warp takes at once, rows of activations shorter and longer than the warps'
+shares, shared experts.  The down kernels (gathered tokens, 16 to 64 MB): at both
+ends, both kernels."""
 import pytest
 import torch
 
@@ -16,9 +18,14 @@ pytestmark = pytest.mark.gpu
     (192, 1024, 128, 8, 0, W.MODE_BATCH),    # on it; 2 activation lines for 8 warps of columns
     (600, 256, 1152, 9, 2, W.MODE_TOPK),     # 18 activation lines for 2 warps, 11 rows a token
     (130, 1152, 640, 16, 0, W.MODE_BATCH),   # 9 warps of columns, the second block partly empty
+    (1024, 1024, 128, 8, 0, W.MODE_BATCH),   # 16 MB of tokens, CTA pairs
+    (910, 1024, 128, 8, 1, W.MODE_TOPK),     # just below
+    (150, 8192, 128, 7, 1, W.MODE_TOPK),     # 18.75 MB with few tokens an expert, shared rows
+    (4096, 1024, 128, 8, 0, W.MODE_TOPK),    # 64 MB
+    (4097, 1024, 128, 8, 0, W.MODE_TOPK),    # just above
 ])
 def test_discard(X, B, d, F, k, n_shared, mode):  # noqa: F811
-    w = W.TINY.with_(B=B, N=24, d=d, F=F, k=k, budget=18, mode=mode)
+    w = W.TINY.with_(B=B, N=24 if d < 8192 else 120, d=d, F=F, k=k, budget=18, mode=mode)
     x, W_g = W.router_inputs(w, seed=4)
     weights = W.expert_weights(w, seed=4, device="cuda")
     shared = W.expert_weights(w.with_(N=n_shared), seed=5, device="cuda") if n_shared else None
