@@ -42,6 +42,7 @@
 #include <atomic>
 #include <cstring>
 
+#include "conv_ring.cuh"
 #include "tc_ptx.cuh"
 #include "tmap.cuh"
 #include "xs_internal.cuh"
@@ -210,13 +211,14 @@ __global__ void __launch_bounds__(kThreads, 1) router_tc_kernel(const __grid_con
   } else if (warp < 2 + 4 * kConvGroups) {
     // ------------------------------------------------ weight planes
     const int cw = (warp - 2) & 3, group = (warp - 2) >> 2;
-    int stage = group % stages;
-    uint32_t phase = static_cast<uint32_t>(group / stages) & 1u;
-    for (int kk = k_begin + group; kk < k_end; kk += kConvGroups) {
-      if (!mbar_wait(full_bar(stage), phase, kWaitNs, abort_flag)) {
+    ConvRing<kConvGroups> ring(group, stages);
+    for (int kk = k_begin + group; kk < k_end; kk += kConvGroups, ring.next()) {
+      if (!ring.wait([&](int s, uint32_t ph) { return mbar_wait(empty_bar(s), ph, kWaitNs, abort_flag); },
+                     [&](int s, uint32_t ph) { return mbar_wait(full_bar(s), ph, kWaitNs, abort_flag); })) {
         *abort_flag = 1;
         break;
       }
+      const int stage = ring.stage;
       const float *wt = reinterpret_cast<const float *>(w_s(stage));
 #pragma unroll
       for (int r = cw; r < kNt; r += 4) {
@@ -239,11 +241,6 @@ __global__ void __launch_bounds__(kThreads, 1) router_tc_kernel(const __grid_con
       }
       fence_proxy_async_smem();
       mbar_arrive(conv_bar(stage));
-      stage += kConvGroups;
-      if (stage >= stages) {
-        stage -= stages;
-        phase ^= 1u;
-      }
     }
   } else {
     // ------------------------------------------------ drain: one fp32 add per stage
@@ -330,6 +327,8 @@ __global__ void __launch_bounds__(kThreads, 1) router_tc_kernel(const __grid_con
 struct RtShape {
   int nt, S, tiles_n, grid, stages;
 };
+
+static_assert(kSmemBudget / stage_bytes(64) >= 2, "ConvRing takes two or more stages");
 
 int stages_for(int nt) {
   const int st = kSmemBudget / stage_bytes(nt);
