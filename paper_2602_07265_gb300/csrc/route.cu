@@ -10,6 +10,7 @@
 #include <climits>
 #include <cmath>
 
+#include "block_sort.cuh"
 #include "xs_internal.cuh"
 
 namespace xs {
@@ -264,31 +265,6 @@ __device__ __forceinline__ void lane_mark_top(const LaneList<Q> &L, int count, M
     if (tie && __popc(b & ((1u << lane) - 1u)) < need) mark(lane_index<Q>(L, q));
     need -= __popc(b);
   }
-}
-
-// Sorts one value per thread in descending order over the first n threads
-// (rounded up to a power of two of at least 32; the others' values do not
-// matter), a bitonic network through shuffles and, between warps, s_x
-// ([blockDim]).  Every thread of the block calls it.
-__device__ __forceinline__ unsigned long long block_sort_desc(unsigned long long v, int n,
-                                                              unsigned long long *s_x) {
-  const int tid = threadIdx.x;
-  for (int k = 2; k < 2 * n || k <= 32; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      unsigned long long o;
-      if (j >= 32) {
-        __syncthreads();
-        s_x[tid] = v;
-        __syncthreads();
-        o = s_x[tid ^ j];
-      } else {
-        o = __shfl_xor_sync(kFull, v, j);
-      }
-      const bool larger = ((tid & j) == 0) == ((tid & k) == 0);
-      v = larger == (v > o) ? v : o;
-    }
-  }
-  return v;
 }
 
 // Halving tree over the expert index of values held as v[q] = value of expert
@@ -1232,6 +1208,7 @@ __global__ void __launch_bounds__(kRouteThreads, 1) score_kernel(RouteArgs a) {
         }
       }
     } else {
+      static_assert(kRouteThreads == kMaxN, "s_masks holds one sorted value per thread");
       unsigned long long *s_sort = reinterpret_cast<unsigned long long *>(s_masks);  // free until the permutation
       if (warp == 0) {
         float vE[kQ], v0[kQ];
@@ -1252,8 +1229,6 @@ __global__ void __launch_bounds__(kRouteThreads, 1) score_kernel(RouteArgs a) {
       const unsigned long long mine =
           live ? (static_cast<unsigned long long>(score_key(s_col[tid])) << 32) | (0xffffffffu - tid) : 0ull;
       const unsigned long long sorted = block_sort_desc(mine, N, s_sort);
-      if (tid < kMaxN) s_sort[tid] = sorted;
-      __syncthreads();
       if (tid == 0) {
         const float target = __int_as_float(s_scal[1]);
         float f = __int_as_float(s_scal[2]);
