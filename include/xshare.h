@@ -406,7 +406,10 @@ void xshare_stack_graph_destroy(xs_graph *g);
  * pipeline wait of the library uses, on a barrier that nothing arrives at.
  * After `budget_ns` nanoseconds (1 .. 2e9) the wait gives up; the kernel
  * writes XS_DEV_TIMEOUT to stats->status, the milliseconds it waited to
- * stats->reserved[0], and returns, leaving the CUDA context usable.
+ * stats->reserved[0], and, after a second wait that runs out for half of the
+ * warp's lanes only, the number of lanes told that it succeeded (0, since all
+ * lanes get one answer) to stats->reserved[1]; it returns after twice the
+ * budget, leaving the CUDA context usable.
  * stats: device pointer (not NULL).  Asynchronous on `stream`. */
 int xshare_selftest_wait_timeout(xs_stats *stats, uint64_t budget_ns, xs_stream_t stream);
 

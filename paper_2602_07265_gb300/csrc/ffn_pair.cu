@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_pair_kernel(const __grid_cons
       const uint32_t bytes = step_bytes(t);
       for (int kk = 0; kk < KI; ++kk, ++i) {
         if (i >= n_pre) {
-          ok = __all_sync(0xffffffffu, mbar_wait(empty_bar(stage), phase ^ 1u, kWaitNs, abort_flag));
+          ok = mbar_wait_warp(empty_bar(stage), phase ^ 1u, kWaitNs, abort_flag);
           if (!ok) break;
         }
         if (elect_one()) {
@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_pair_kernel(const __grid_cons
     // The last MMAs have read every stage, and this CTA got every signal that
     // is sent to it.
     for (int j = 0; ok && j < kStages; ++j) {
-      ok = __all_sync(0xffffffffu, mbar_wait(empty_bar(stage), phase ^ 1u, kWaitNs, abort_flag));
+      ok = mbar_wait_warp(empty_bar(stage), phase ^ 1u, kWaitNs, abort_flag);
       if (++stage == kStages) {
         stage = 0;
         phase ^= 1u;
@@ -294,12 +294,12 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_pair_kernel(const __grid_cons
         const Unit t = unit_at(u, false);
         const uint32_t idesc = __shfl_sync(0xffffffffu, idesc_bf16(256, t.n_mma), 0);
         const int buf = seq & 1;
-        ok = __all_sync(0xffffffffu, mbar_wait(accempty_bar(buf), ((seq >> 1) & 1u) ^ 1u, kWaitNs, abort_flag));
+        ok = mbar_wait_warp(accempty_bar(buf), ((seq >> 1) & 1u) ^ 1u, kWaitNs, abort_flag);
         if (!ok) break;
         tc_fence_after();
         const uint32_t d0 = acc0 + buf * kAccCols;
         for (int kk = 0; kk < KI; ++kk) {
-          ok = __all_sync(0xffffffffu, mbar_wait(full_bar(stage), phase, kWaitNs, abort_flag));
+          ok = mbar_wait_warp(full_bar(stage), phase, kWaitNs, abort_flag);
           if (!ok) break;
           tc_fence_after();
           const uint64_t da = desc0 + static_cast<uint64_t>(stage * (kStageBytes >> 4));
@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_pair_kernel(const __grid_cons
       // All issued MMAs done before TMEM is released.
       if (elect_one()) mma_commit_pair_local(drain_bar);
       volatile int no_abort = 0;
-      mbar_wait(drain_bar, 0, kWaitNs, &no_abort);
+      mbar_wait_warp(drain_bar, 0, kWaitNs, &no_abort);
     } else if (!kGateUp && p.drop != nullptr) {
       // The rows of all tiles, in equal shares over the pairs that have work.
       const Unit a = unit_at(0, false), b = unit_at(n_units - 1, false);
@@ -343,11 +343,10 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_pair_kernel(const __grid_cons
     for (int u = pair; u < n_units; u += n_pairs, ++seq) {
       const Unit t = unit_at(u, false);
       const int buf = seq & 1;
-      if (!mbar_wait(accfull_bar(buf), (seq >> 1) & 1u, kWaitNs, abort_flag)) {
+      if (!mbar_wait_warp(accfull_bar(buf), (seq >> 1) & 1u, kWaitNs, abort_flag)) {
         if (lane == 0) fail();
         break;
       }
-      __syncwarp();
       tc_fence_after();
       const uint32_t tacc = tmem + (static_cast<uint32_t>(q * 32) << 16) + buf * kAccCols;
       const int n_cols = rows_of(t, rank) ? t.n_mma : 0;   // columns this CTA finishes

@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_tc_kernel(const __grid_consta
     for (long long it = it_begin + n_pre; it < it_end; ++it, advance(c)) {
       source(c, r, false);
       const int kk = c.kk;
-      ok = __all_sync(0xffffffffu, mbar_wait(empty_bar(stage), phase ^ 1u, kWaitNs, abort_flag));
+      ok = mbar_wait_warp(empty_bar(stage), phase ^ 1u, kWaitNs, abort_flag);
       if (!ok) break;
       if (elect_one()) {
         const uint32_t sA = sbase + stage * C::kStageBytes;
@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_tc_kernel(const __grid_consta
     // Never leave with copies in flight: wait (bounded) for the last load of every stage.
     volatile int no_abort = 0;
     for (int s = 0; s < C::kStages; ++s)
-      if ((issued_mask >> s) & 1u) mbar_wait(full_bar(s), (issued_phase >> s) & 1u, kWaitNs, &no_abort);
+      if ((issued_mask >> s) & 1u) mbar_wait_warp(full_bar(s), (issued_phase >> s) & 1u, kWaitNs, &no_abort);
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer
     const uint32_t base = __shfl_sync(0xffffffffu, sbase, 0), acc0 = __shfl_sync(0xffffffffu, tmem, 0);
@@ -376,12 +376,12 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_tc_kernel(const __grid_consta
       const uint32_t idesc = __shfl_sync(0xffffffffu, idesc_bf16(kBM, n_mma), 0);
       const int buf = segi & 1;
       const uint32_t use = static_cast<uint32_t>(segi >> 1);
-      ok = __all_sync(0xffffffffu, mbar_wait(accempty_bar(buf), (use & 1u) ^ 1u, kWaitNs, abort_flag));
+      ok = mbar_wait_warp(accempty_bar(buf), (use & 1u) ^ 1u, kWaitNs, abort_flag);
       if (!ok) break;
       tc_fence_after();
       const uint32_t d0 = acc0 + buf * C::kAccCols;
       for (int kk = k0; kk < k1; ++kk) {
-        ok = __all_sync(0xffffffffu, mbar_wait(full_bar(stage), phase, kWaitNs, abort_flag));
+        ok = mbar_wait_warp(full_bar(stage), phase, kWaitNs, abort_flag);
         if (!ok) break;
         tc_fence_after();
         const uint32_t sA = base + stage * C::kStageBytes;
@@ -412,7 +412,7 @@ __global__ void __launch_bounds__(kThreads, 1) ffn_tc_kernel(const __grid_consta
     if (any) {  // all issued MMAs done before TMEM is released
       volatile int no_abort = 0;
       if (elect_one()) mma_commit(drain_bar);
-      mbar_wait(drain_bar, 0, kWaitNs, &no_abort);
+      mbar_wait_warp(drain_bar, 0, kWaitNs, &no_abort);
     }
   } else {
     // ------------------------------------------------ epilogue (warps 2..5)

@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(kThreads, 1) router_tc_kernel(const __grid_con
     int stage = 0;
     uint32_t phase = 0, issued_mask = 0, issued_phase = 0;
     for (int kk = k_begin; kk < k_end; ++kk) {
-      if (!__all_sync(0xffffffffu, mbar_wait(empty_bar(stage), phase ^ 1u, kWaitNs, abort_flag))) {
+      if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, kWaitNs, abort_flag)) {
         *abort_flag = 1;
         break;
       }
@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kThreads, 1) router_tc_kernel(const __grid_con
     // Never leave with copies in flight: wait (bounded) for the last load of every stage.
     volatile int no_abort = 0;
     for (int s = 0; s < stages; ++s)
-      if ((issued_mask >> s) & 1u) mbar_wait(full_bar(s), (issued_phase >> s) & 1u, kWaitNs, &no_abort);
+      if ((issued_mask >> s) & 1u) mbar_wait_warp(full_bar(s), (issued_phase >> s) & 1u, kWaitNs, &no_abort);
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer
     const uint32_t idesc = idesc_bf16(kBM, kNt);
@@ -176,9 +176,8 @@ __global__ void __launch_bounds__(kThreads, 1) router_tc_kernel(const __grid_con
     for (int kk = k_begin; kk < k_end; ++kk) {
       const int i = kk - k_begin, buf = i % kBufs;
       const uint32_t use = static_cast<uint32_t>(i / kBufs);
-      const bool ready = mbar_wait(conv_bar(stage), phase, kWaitNs, abort_flag) &&
-                         mbar_wait(acce_bar(buf), (use & 1u) ^ 1u, kWaitNs, abort_flag);
-      if (!__all_sync(0xffffffffu, ready)) {
+      if (!mbar_wait_warp(conv_bar(stage), phase, kWaitNs, abort_flag) ||
+          !mbar_wait_warp(acce_bar(buf), (use & 1u) ^ 1u, kWaitNs, abort_flag)) {
         *abort_flag = 1;
         break;
       }
@@ -206,15 +205,15 @@ __global__ void __launch_bounds__(kThreads, 1) router_tc_kernel(const __grid_con
     if (any) {  // all issued MMAs done before TMEM is released
       volatile int no_abort = 0;
       if (elect_one()) mma_commit(drain_bar);
-      mbar_wait(drain_bar, 0, kWaitNs, &no_abort);
+      mbar_wait_warp(drain_bar, 0, kWaitNs, &no_abort);
     }
   } else if (warp < 2 + 4 * kConvGroups) {
     // ------------------------------------------------ weight planes
     const int cw = (warp - 2) & 3, group = (warp - 2) >> 2;
     ConvRing<kConvGroups> ring(group, stages);
     for (int kk = k_begin + group; kk < k_end; kk += kConvGroups, ring.next()) {
-      if (!ring.wait([&](int s, uint32_t ph) { return mbar_wait(empty_bar(s), ph, kWaitNs, abort_flag); },
-                     [&](int s, uint32_t ph) { return mbar_wait(full_bar(s), ph, kWaitNs, abort_flag); })) {
+      if (!ring.wait([&](int s, uint32_t ph) { return mbar_wait_warp(empty_bar(s), ph, kWaitNs, abort_flag); },
+                     [&](int s, uint32_t ph) { return mbar_wait_warp(full_bar(s), ph, kWaitNs, abort_flag); })) {
         *abort_flag = 1;
         break;
       }
@@ -251,7 +250,7 @@ __global__ void __launch_bounds__(kThreads, 1) router_tc_kernel(const __grid_con
     for (int kk = k_begin; kk < k_end; ++kk) {
       const int i = kk - k_begin, buf = i % kBufs;
       const uint32_t use = static_cast<uint32_t>(i / kBufs);
-      if (!mbar_wait(accf_bar(buf), use & 1u, kWaitNs, abort_flag)) {
+      if (!mbar_wait_warp(accf_bar(buf), use & 1u, kWaitNs, abort_flag)) {
         *abort_flag = 1;
         break;
       }

@@ -64,6 +64,16 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint64_
   }
 }
 
+// The same for the whole warp, which gets one answer: true if every lane's
+// wait ended.  Near a timeout or an abort the lanes, each with its own clock
+// and its own read of *abort, can differ; a warp that split there would leave
+// lanes behind in the next warp-wide instruction (shuffles, TMEM loads,
+// barriers), for good.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, uint64_t budget_ns,
+                                               volatile int *abort) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, budget_ns, abort));
+}
+
 // ---------------------------------------------------------------- TMA
 
 __device__ __forceinline__ uint64_t policy_evict_first() {

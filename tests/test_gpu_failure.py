@@ -49,6 +49,14 @@ def test_bounded_wait_reports_timeout_and_context_survives(X):
     assert torch.isfinite(y.float()).all()
 
 
+def test_all_lanes_of_a_warp_get_one_answer(X):
+    # A wait that runs out for the even lanes and ends in time for the odd ones.
+    st = torch.full((X.STATS_WORDS,), -1, dtype=torch.int32, device="cuda")
+    X.xshare_selftest_wait_timeout(st, 20_000_000)
+    torch.cuda.synchronize()
+    assert st.cpu().tolist()[7] == 0
+
+
 def test_selftest_rejects_bad_budget(X):
     st = torch.zeros(X.STATS_WORDS, dtype=torch.int32, device="cuda")
     with pytest.raises(X.XShareError):
