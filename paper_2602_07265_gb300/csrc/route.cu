@@ -1812,6 +1812,8 @@ static cudaError_t launch_scatter(const RouteArgs &a, cudaStream_t s) {
                     reinterpret_cast<const int32_t *>(a.chunk_col), a.perm_out, P, a.N, a.k);
 }
 
+static_assert(kScoreRowBytes >= kChunk * kMaxN * 4, "score_kernel always has a chunk's rows");
+
 template <int kQ>
 cudaError_t launch_route_q(const RouteArgs &a, cudaStream_t s) {
   const int C = (a.B + kChunk - 1) / kChunk;
@@ -1829,7 +1831,10 @@ cudaError_t launch_route_q(const RouteArgs &a, cudaStream_t s) {
   const int need = a.mode != XS_MODE_HIER || a.T > kChunk ? 0 : kChunk % a.T == 0 ? kChunk : kChunk + a.T - 1;
   b.hier_rows = need * a.N * 4 <= kScoreRowBytes ? need : 0;
   const int dyn1 = (b.hier_rows > kChunk ? b.hier_rows : kChunk) * a.N * 4;
-  e = cudaFuncSetAttribute(score_kernel<kQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn1);
+  // The most that any call needs, not dyn1: the attribute belongs to the
+  // kernel, and a host thread with a smaller call would lower it between
+  // another thread's setting and launch, which then fails.
+  e = cudaFuncSetAttribute(score_kernel<kQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, kScoreRowBytes);
   if (e != cudaSuccess) return e;
   e = launch_pdl(score_kernel<kQ>, dim3(2 * C), dim3(kRouteThreads), (size_t)dyn1, s, b);
   if (e != cudaSuccess) return e;

@@ -236,9 +236,11 @@ cudaError_t launch_rs(const uint16_t *x, const float *Wg, float *h, int B, int N
   const int nch = d / kRsChunk;
   const int DSmax = ((nch + S - 1) / S) * kRsChunk;
   const size_t smem = rs_smem_bytes(DSmax, rs_tb(kTI));
+  // The most that any d needs (see launch_route_q): calls of other host
+  // threads must not lower it.
   cudaError_t e = cudaFuncSetAttribute(router_split_kernel<kTI>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+                                       static_cast<int>(rs_smem_bytes(kRsMaxDS, rs_tb(kTI))));
   if (e != cudaSuccess) return e;
   dim3 grid((N + kRsEB - 1) / kRsEB, S, (B + rs_tb(kTI) - 1) / rs_tb(kTI));
   return launch_pdl(router_split_kernel<kTI>, grid, dim3(kRsThreads), smem, s, x, Wg, h, B, N, d,
