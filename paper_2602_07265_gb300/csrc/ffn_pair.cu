@@ -84,13 +84,6 @@ struct PairParams {
   int expert_base;      // routed expert e uses weights e - expert_base (expert parallelism)
 };
 
-// g / (1 + exp(-g)) from t = exp(-|g|): the denominator 1 + t lies in [1, 2],
-// where the fast division is accurate to 2 ulp.
-__device__ __forceinline__ float silu(float g) {
-  const float t = expf(-fabsf(g));
-  return __fdividef(g >= 0.f ? g : g * t, 1.f + t);
-}
-
 template <bool kGateUp>
 __global__ void __launch_bounds__(kThreads, 1) ffn_pair_kernel(const __grid_constant__ PairParams p) {
   extern __shared__ uint8_t smem_raw[];

@@ -124,8 +124,6 @@ __device__ __forceinline__ void set_status(const TcParams &p, int code) {
   if (p.stats) atomicMax(&p.stats->status, code);
 }
 
-__device__ __forceinline__ float silu(float g) { return g / (1.f + expf(-g)); }
-
 template <bool kGateUp>
 __global__ void __launch_bounds__(kThreads, 1) ffn_tc_kernel(const __grid_constant__ TcParams p) {
   using C = Cfg<kGateUp>;

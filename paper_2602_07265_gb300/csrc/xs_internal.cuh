@@ -43,6 +43,9 @@ cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, size_t 
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
+// Both FFN paths round alike: a correctly rounded division.
+__device__ __forceinline__ float silu(float g) { return g / (1.f + expf(-g)); }
+
 // Drops the 128-byte line at p (aligned) from L2 without writing it back.
 __device__ __forceinline__ void discard_line(const void *p) {
   asm volatile("discard.global.L2 [%0], 128;" ::"l"(p) : "memory");

@@ -41,6 +41,20 @@ def test_pair_forward(X, N, k, d, F, B, mode, n_shared):  # noqa: F811
     assert torch.equal(y.cpu().double(), torch.from_numpy(g["y"])), "packed and plain weights differ"
 
 
+def test_pair_rounds_like_the_other_path(X):  # noqa: F811
+    """A token's output does not depend on the path: 8 experts of 18 blocks are
+    whole units on either (ffn_tc.cu gives each of 144 CTAs one), so that a
+    batch of 7 tokens, which ffn_tc.cu takes, has the bits of the same tokens
+    in a batch of 256, which the pairs take."""
+    w = W.TINY.with_(N=8, k=8, d=2304, F=2304, B=256, mode=W.MODE_TOPK, budget=0, k0=0)
+    x, W_g, weights, _ = _inputs(w, 0)
+    pk = X.Packed(*weights)
+    y = run_one_gpu(X, w, x, W_g, pk)["y"]
+    for t in range(0, w.B - 7, 7):
+        few = run_one_gpu(X, w.with_(B=7), x[t:t + 7].contiguous(), W_g, pk)["y"]
+        assert torch.equal(few, y[t:t + 7])
+
+
 def test_pair_expert_parallel(X):  # noqa: F811
     w = W.TINY.with_(N=8, k=2, d=256, F=256, B=900, mode=W.MODE_TOPK, x_kind="domains")
     x, W_g, weights, shared = _inputs(w, 1)
