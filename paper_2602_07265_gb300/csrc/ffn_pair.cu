@@ -47,6 +47,7 @@
 #include <atomic>
 #include <cstring>
 
+#include "pair_rule.cuh"
 #include "tc_ptx.cuh"
 #include "tmap.cuh"
 #include "xs_internal.cuh"
@@ -504,19 +505,8 @@ cudaError_t launch_phase(const FfnArgs &a, cudaStream_t s) {
 
 }  // namespace
 
-bool ffn_use_pairs(long long pairs, int experts, int d, int F) {
-  const int P = resident_pairs();
-  if (P <= 0 || experts <= 0) return false;
-  if (pairs >= static_cast<long long>(kPairMinTok) * experts) return true;
-  if (pairs < static_cast<long long>(kPairFewTok) * experts &&
-      pairs * d < static_cast<long long>(kPairWork) * experts)
-    return false;
-  // Rounds that the whole units take, against the time their work would fill.
-  auto idles = [&](double blocks, int units) {
-    const long long rounds = (static_cast<long long>(experts) * units + P - 1) / P;
-    return static_cast<double>(rounds) * P > experts * blocks * (1.0 + kPairIdle);
-  };
-  return !idles(F / 128.0, F / 128) && !idles(d / 256.0, (d + 255) / 256);
+bool ffn_use_pairs(long long pairs, int experts, int ranks, int d, int F) {
+  return pair_rule(pairs, experts, (experts + ranks - 1) / ranks, resident_pairs(), d, F);
 }
 
 cudaError_t launch_ffn_pair_gate_up(const FfnArgs &a, cudaStream_t s) { return launch_phase<true>(a, s); }

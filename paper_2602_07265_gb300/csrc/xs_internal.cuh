@@ -102,27 +102,6 @@ __host__ __device__ inline int ffn_ctas(long long U, int KI, int grid) {
   return static_cast<int>(want < grid ? want : grid);
 }
 
-// When a batch takes the CTA-pair FFN kernels (ffn_pair.cu), by its pairs per
-// expert that can be selected (T):
-//   - always from kPairMinTok on;
-//   - from kPairFewTok on, or from T K >= kPairWork (long units hide a unit's
-//     fixed costs), if neither phase idles more than kPairIdle of its time in
-//     the last round of units, or on the missing half of an odd down block.
-// Layer forward on GB300, plain top-k, ffn_tc.cu | ffn_pair.cu, us:
-//   N = 64, d = 2048, F = 1024 (3.9 % idle): T = 8 142.1 | 143.5, 12.5 144.4 |
-//   141.1, 24 149.2 | 145.5, 64 172.1 | 155.0, 128 277.9 | 179.1
-//   N = 128, d = 2048, F = 768 (8.9 %): T = 8 201.4 | 203.1, 16 208.1 | 211.4,
-//   24 213.4 | 211.2, 32 223.1 | 217.6, 128 405.1 | 285.3
-//   N = 16, d = 5120, F = 2048 (18.7 %): T = 19 171.2 | 176.0, 37 179.9 | 180.3
-//   N = 300, d = 640, F = 1920 (21 % in the down phase): T = 15 361.9 | 367.3
-//   N = 256, d = 7168, F = 2048, budget 24, k0 = 1: B = 32 (T = 4.6) 552 | 561,
-//   B = 64 (5.8) 739 | 727, B = 96 (6.4) 858 | 838, B = 128 (6.7) 950 | 938;
-//   groups, B = 256 (8) 772 | 763
-constexpr int kPairMinTok = 24;
-constexpr int kPairFewTok = 12;
-constexpr int kPairWork = 600 * 64;
-constexpr double kPairIdle = 0.045;
-
 // One FFN work tile: up to kTileTok (kPairTok) consecutive rows of the permuted pair
 // list, all routed to `expert`.  Experts N .. N + n_shared - 1 are the shared
 // experts; their rows follow the routed pairs: row n_pairs + j * B + t is
@@ -292,8 +271,9 @@ struct FfnArgs {
 cudaError_t launch_ffn_gate_up(const FfnArgs &a, cudaStream_t s);
 cudaError_t launch_ffn_down(const FfnArgs &a, cudaStream_t s);
 // The same on CTA pairs, for tiles of up to kPairTok tokens; whether a batch of
-// `pairs` routed pairs over at most `experts` experts takes them.
-bool ffn_use_pairs(long long pairs, int experts, int d, int F);
+// `pairs` routed pairs over at most `experts` experts takes them (pair_rule.cuh),
+// a layer split over `ranks` GPUs on each of them.
+bool ffn_use_pairs(long long pairs, int experts, int ranks, int d, int F);
 cudaError_t launch_ffn_pair_gate_up(const FfnArgs &a, cudaStream_t s);
 cudaError_t launch_ffn_pair_down(const FfnArgs &a, cudaStream_t s);
 size_t ffn_part_bytes(int n_sms);

@@ -27,7 +27,10 @@ def _inputs(w, n_shared):
     (2, 2, 256, 384, 256, W.MODE_TOPK, 1), (3, 3, 640, 128, 257, W.MODE_TOPK, 0),
     (8, 2, 256, 256, 1000, W.MODE_TOPK, 2), (32, 4, 128, 384, 700, W.MODE_BATCH, 0),
     (16, 3, 2048, 256, 513, W.MODE_HIER, 0), (2, 2, 512, 128, 30, W.MODE_TOPK, 0),
-    (38, 8, 512, 256, 63, W.MODE_TOPK, 1), (38, 4, 512, 256, 150, W.MODE_TOPK, 0)])
+    (38, 8, 512, 256, 63, W.MODE_TOPK, 1), (38, 4, 512, 256, 150, W.MODE_TOPK, 0),
+    # few experts, long units (112 steps on 8 of the pairs; two rounds of 112), and the other side of the rule
+    (4, 2, 7168, 256, 64, W.MODE_TOPK, 0), (4, 2, 7168, 2560, 100, W.MODE_TOPK, 0),
+    (4, 2, 7168, 256, 48, W.MODE_TOPK, 0)])
 def test_pair_forward(X, N, k, d, F, B, mode, n_shared):  # noqa: F811
     w = W.TINY.with_(N=N, k=k, d=d, F=F, B=B, mode=mode, budget=6, k0=0, m_r=2,
                      tokens_per_request=3 if mode == W.MODE_HIER else 1, x_kind="domains")

@@ -1,0 +1,60 @@
+"""The rule that sends a batch to the CTA-pair FFN kernels (pair_rule.cuh), on
+the CPU: the side that measured faster on GB300 (76 pairs at once) at layers
+of few experts, of narrow experts and of long units."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2602_07265_gb300", "csrc")
+
+MAIN = r"""
+#include <cstdio>
+#include <cstdlib>
+#include "pair_rule.cuh"
+int main(int argc, char **argv) {
+  int v[6];
+  for (int i = 0; i < 6; ++i) v[i] = std::atoi(argv[1 + i]);
+  std::puts(xs::pair_rule(v[0], v[1], v[2], v[3], v[4], v[5]) ? "1" : "0");
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def rule(tmp_path_factory):
+    if shutil.which("g++") is None:
+        pytest.skip("needs g++")
+    d = tmp_path_factory.mktemp("pair_rule")
+    (d / "rule.cpp").write_text(MAIN)
+    exe = d / "rule"
+    subprocess.run(["g++", "-std=c++17", "-I" + CSRC, str(d / "rule.cpp"), "-o", str(exe)], check=True)
+
+    def run(T, N, d, F, here=None, P=76):
+        args = [T * N, N, N if here is None else here, P, d, F]
+        return subprocess.run([str(exe)] + [str(a) for a in args], capture_output=True, text=True,
+                              check=True).stdout.strip() == "1"
+    return run
+
+
+@pytest.mark.parametrize("T,N,d,F,pairs", [
+    # Several rounds of units whose last one leaves the pairs idle for long.
+    (24, 16, 5120, 2048, False), (32, 16, 5120, 2048, False), (48, 16, 5120, 2048, True),
+    (24, 300, 640, 1920, False), (32, 300, 640, 1920, False), (64, 300, 640, 1920, True),
+    (24, 16, 6144, 1408, False), (32, 16, 6144, 1408, False), (48, 16, 6144, 1408, True),
+    (24, 16, 7168, 2048, False), (64, 16, 7168, 2048, True),
+    # One round of long units on few SMs: a loss at 24 tokens, a gain at 32.
+    (24, 4, 7168, 256, False), (32, 4, 7168, 256, True), (24, 8, 7168, 256, True),
+    # Few or narrow experts that gain.
+    (24, 8, 2048, 256, True), (24, 4, 2048, 2048, True), (24, 8, 7168, 1024, True), (24, 32, 2048, 256, True),
+    (24, 64, 1024, 512, True), (24, 64, 2048, 1024, True), (24, 32, 7168, 2048, True), (24, 5, 1280, 640, True),
+    # Below 24 tokens: by the share of idle time.
+    (12, 64, 2048, 1024, True), (8, 64, 2048, 1024, False), (16, 128, 2048, 768, False)])
+def test_side_that_measured_faster(rule, T, N, d, F, pairs):
+    assert rule(T, N, d, F) == pairs
+
+
+def test_a_rank_counts_its_own_units(rule):
+    # 55 experts of 16 blocks fill whole rounds on one GPU; a rank's seven do not.
+    assert rule(8, 55, 7168, 2048) and not rule(8, 55, 7168, 2048, here=7)
+    assert not rule(64, 8, 2048, 256, P=0)   # the kernels cannot run
