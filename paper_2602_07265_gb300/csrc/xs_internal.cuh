@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <utility>
 
+#include "router_rule.cuh"
 #include "xshare.h"
 
 namespace xs {
@@ -189,24 +190,6 @@ struct RouteArgs {
 cudaError_t launch_route(const RouteArgs &a, cudaStream_t s);
 // Clears the arrival counters done[0 .. 3] for a launch_route that follows.
 cudaError_t launch_clear(int32_t *done, cudaStream_t s);
-// Which router a batch takes.  The tensor cores' costs about 9 us whatever the
-// batch; the CUDA cores' grows with the work.  Below 64 tokens the latter
-// always wins; for narrow layers (d < kRouterSplitMinD) up to B N d of about
-// kRouterFmas.  Layer forward on GB300, plain top-k, tensor | CUDA cores, us:
-//   d = 2048: N = 64, B = 150 (20 M) 67.3 | 64.3, 250 (33 M) 68.5 | 67.6, 350
-//   (46 M) 68.9 | 69.4; N = 256, B = 64 (34 M) 101.2 | 98.9, 100 (52 M) 92.7 | 93.2
-//   d = 1024, N = 64: B = 300 (20 M) 51.8 | 49.6, 1000 (66 M) 60.1 | 62.9
-//   d = 512, N = 512: B = 64 (17 M) 82.6 | 81.3, 128 (34 M) 72.5 | 76.6
-//   d = 3072, N = 128: B = 64 (25 M) 88.4 | 86.9, 128 (50 M) 85.1 | 86.1
-// (The CUDA cores' sums are the more exact ones: largest relative error of a
-// score against 64 bits 1.0 to 1.4e-6, the tensor cores' 3.0 to 3.5e-6.)
-constexpr int kRouterTcMinB = 64;
-constexpr long long kRouterFmas = 32ll << 20;
-constexpr int kRouterSplitMinD = 4096;
-constexpr int kRouterSplitMaxD = 16384;
-inline bool router_on_tensor_cores(int B, int N, int d) {
-  return B >= kRouterTcMinB && (d >= kRouterSplitMinD || static_cast<long long>(B) * N * d > kRouterFmas);
-}
 // Router logits on the CUDA cores (see router_on_tensor_cores).  d outside
 // [kRouterSplitMinD, kRouterSplitMaxD]: whole-d blocks of 8 tokens x 4 experts (route.cu),
 // h[t][e].  d inside: d-sliced blocks (router_split.cu), h[s][t][e] for s <

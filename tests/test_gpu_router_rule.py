@@ -13,6 +13,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("N,d,B", [
     (64, 2048, 63), (64, 2048, 64), (64, 2048, 256), (64, 2048, 257), (100, 512, 655), (100, 512, 656),
     (8, 3968, 1057), (8, 3968, 1058), (9, 4096, 64), (1024, 128, 256), (1024, 128, 257),
+    (128, 128, 192), (128, 128, 193), (32, 256, 768), (32, 256, 769), (16, 2048, 1024), (16, 2048, 1025),
     (66, 512, 3000), (130, 512, 8191), (132, 512, 8191)])
 def test_both_routers(X, N, d, B):  # noqa: F811
     w = W.TINY.with_(N=N, d=d, F=128, B=B, k=4, budget=6)
