@@ -238,8 +238,8 @@ int xshare_moe_forward(const uint16_t *x, const float *W_g, const uint16_t *W_ga
  *   - every call on a device uses the same array, so calls that can overlap
  *     on the GPU (different streams, or different host threads) race and
  *     must be ordered by the caller.  Each call clears the three arrival
- *     counters it keeps in the array (a small kernel on `stream`); every
- *     other scratch word is written before it is read.
+ *     counters and the flag it keeps in the array (a small kernel on
+ *     `stream`); every other scratch word is written before it is read.
  * Allocates nothing (no cudaMalloc, cudaFree or allocating library call). */
 int xshare_route_static(const float *scores, int B, int N, int k, int budget, int mode,
                         const xs_route_params *prm, uint8_t *sel_mask, int32_t *topk_ids,

@@ -16,14 +16,14 @@
 //   - two 256-column TMEM accumulators let the epilogue of a unit run under
 //     the MMAs of the next.
 // Measured on GB300 (whole layer, ffn_tc.cu -> this): d = 2048, F = 1024, 48
-// experts, B = 8192 (1365 tokens an expert) 1479 -> 725 us (gate/up 829 -> 335
-// us, 1.64 PFLOP/s; down 436 -> 213 us, which also writes 537 MB of fp32 rows:
+// experts, B = 8192 (1365 tokens an expert) 1452 -> 702 us (gate/up 820 -> 333
+// us, 1.65 PFLOP/s; down 440 -> 211 us, which also writes 537 MB of fp32 rows:
 // 178 us without the stores); d = 2048, F = 768, 128 experts, B = 2048 (128
-// tokens) 416 -> 284 us (gate/up 142 us for 805 MB of weights).  Four
+// tokens) 394 -> 278 us (gate/up 143 us for 805 MB of weights).  Four
 // pipeline stages instead of six cost 5 %, tiles dealt expert by expert to all
 // pairs (one row block at a time) 19 %.  With the loads left out the MMAs and
 // the epilogue of the first case's gate/up phase take 254 us (2.2 PFLOP/s), of
-// the second's 68 us.
+// the second's 68 us (both with a faster, less exact silu; see silu()).
 //
 // Unit: (tile of up to 256 tokens of one expert, block of weight rows).  The
 // weights are the MMA's M = 256 rows, 128 in each CTA; the tokens are its N

@@ -1179,7 +1179,9 @@ __global__ void __launch_bounds__(kRouteThreads, 1) score_kernel(RouteArgs a) {
     // whose lists are not sorted, the block sorts the candidates once (one per
     // thread) and one thread adds their scores in that order.  Routing on
     // GB300, lists | sort: N = 128, B = 64, tau = 0.7 18.4 | 19.4 us, N = 256
-    // 21.6 | 22.4, N = 800 106 | 58.0; N = 400, B = 2000, tau = 0.5 44.1 | 38.2.
+    // 21.6 | 22.4; N = 512, B = 64 79.1 | 40.5, N = 800 159.7 | 61.5, N = 1024,
+    // B = 1000 60.3 | 51.7; N = 400, B = 2000, whose warm-up sets leave nothing
+    // to add, 36.4 | 40.8.
     if constexpr (kQ <= kSortedQ) {
       if (warp == 0) {
         float vE[kQ], v0[kQ];
@@ -1737,10 +1739,12 @@ __global__ void __launch_bounds__(256) combine_kernel(const float *out, const ui
   __shared__ int32_t s_kp, s_pairs;
   const int t = blockIdx.y;
   const int c4 = blockIdx.x * blockDim.x + threadIdx.x;
-  // Before pdl_wait(): the token's rows and weights and the pair count,
-  // written by the routing kernels four launches earlier (complete before
-  // this grid started), and x_t (an input, or the previous layer's output);
-  // only `out` comes from the kernel just before.
+  // Before pdl_wait(): the token's weights and the pair count, written by the
+  // routing kernels, its rows, whose final values the gather kernel writes
+  // for more than kFuseChunks chunks (three launches earlier: gate/up and
+  // down lie between, and gate/up was complete before this grid started), and
+  // x_t (an input, or the previous layer's output); only `out` comes from the
+  // kernel just before.
   if (threadIdx.x < kMaxK) {
     const int s = threadIdx.x;
     s_row[s] = s < k ? __ldcg(pos + (size_t)t * k + s) : -1;

@@ -176,8 +176,8 @@ extern "C" int xshare_route_static(const float *scores, int B, int N, int k, int
   a.tile_tok = kTileTok;
   a.zero_words = nullptr;
   a.zero_count = 0;
-  // The three arrival counters must start at zero; every other scratch word is
-  // written before it is read.
+  // The three arrival counters must start at zero (the flag after them is
+  // cleared too); every other scratch word is written before it is read.
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (launch_clear(a.done, s) != cudaSuccess) return XS_ERR_CUDA;
   return launch_route(a, s) == cudaSuccess ? XS_OK : XS_ERR_CUDA;
