@@ -272,7 +272,8 @@ int xs::forward_impl(const FwdCall &c, FwdStep step) {
   a.zero_words = at<int32_t>(workspace, pl.ffn_cnt);
   a.zero_count = (int)ffn_cnt_words(pl.max_tiles, B, d, F);
   a.n_shared = n_shared;
-  const bool ffn_pairs = ffn_use_pairs(static_cast<long long>(B) * k, max_selected(a), ep ? c.ep_ranks : 1, d, F);
+  const bool ffn_pairs = ffn_use_pairs(static_cast<long long>(B) * k, max_selected(a), c.mode == XS_MODE_TOPK,
+                                       ep ? c.ep_ranks : 1, d, F);
   if (ffn_pairs) a.tile_tok = kPairTok;
 
   FfnArgs f;

@@ -505,8 +505,8 @@ cudaError_t launch_phase(const FfnArgs &a, cudaStream_t s) {
 
 }  // namespace
 
-bool ffn_use_pairs(long long pairs, int experts, int ranks, int d, int F) {
-  return pair_rule(pairs, experts, (experts + ranks - 1) / ranks, resident_pairs(), d, F);
+bool ffn_use_pairs(long long pairs, int experts, bool all, int ranks, int d, int F) {
+  return pair_rule(pairs, experts, (experts + ranks - 1) / ranks, all || ranks == 1, resident_pairs(), d, F);
 }
 
 cudaError_t launch_ffn_pair_gate_up(const FfnArgs &a, cudaStream_t s) { return launch_phase<true>(a, s); }

@@ -46,8 +46,13 @@ constexpr int kPairWork = 600 * 64;
 constexpr double kPairIdle = 0.045;
 
 // `pairs` routed pairs over at most `experts` experts, `here` of them on this
-// GPU; P CTA pairs run at once (0: the kernels cannot run).
-inline bool pair_rule(long long pairs, int experts, int here, int P, int d, int F) {
+// GPU, which for a rank's share of a selection is a guess (`sure` false): below
+// kPairMinTok a rank then stays on ffn_tc.cu, since what pairs gain there is
+// less than a round that the guess misses (N = 256, d = 7168, F = 2048, groups,
+// B = 256, a rank of eight with 32 of the 256 experts that the bound allows and
+// about 8 used: 326.5 | 336.8 us; plain top-k, B = 512, all 32 used: 493 | 467).
+// P CTA pairs run at once (0: the kernels cannot run).
+inline bool pair_rule(long long pairs, int experts, int here, bool sure, int P, int d, int F) {
   if (P <= 0 || experts <= 0) return false;
   auto tokens = [&](int t) { return pairs >= static_cast<long long>(t) * experts; };
   if (tokens(kPairAllTok)) return true;
@@ -69,6 +74,7 @@ inline bool pair_rule(long long pairs, int experts, int here, int P, int d, int 
         (gate_up.rounds > 1 ? gate_up.waited() : 0.0) + (down.rounds > 1 ? down.waited() : 0.0);
     return several <= kPairWait && (tokens(kPairWaitTok) || gate_up.waited() + down.waited() <= kPairWaitAny);
   }
+  if (!sure) return false;
   if (!tokens(kPairFewTok) && pairs * d < static_cast<long long>(kPairWork) * experts) return false;
   return !gate_up.idles() && !down.idles();
 }

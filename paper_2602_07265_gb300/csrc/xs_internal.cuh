@@ -258,9 +258,10 @@ struct FfnArgs {
 cudaError_t launch_ffn_gate_up(const FfnArgs &a, cudaStream_t s);
 cudaError_t launch_ffn_down(const FfnArgs &a, cudaStream_t s);
 // The same on CTA pairs, for tiles of up to kPairTok tokens; whether a batch of
-// `pairs` routed pairs over at most `experts` experts takes them (pair_rule.cuh),
-// a layer split over `ranks` GPUs on each of them.
-bool ffn_use_pairs(long long pairs, int experts, int ranks, int d, int F);
+// `pairs` routed pairs over at most `experts` experts (all: every expert of the
+// layer) takes them (pair_rule.cuh), a layer split over `ranks` GPUs on each of
+// them.
+bool ffn_use_pairs(long long pairs, int experts, bool all, int ranks, int d, int F);
 cudaError_t launch_ffn_pair_gate_up(const FfnArgs &a, cudaStream_t s);
 cudaError_t launch_ffn_pair_down(const FfnArgs &a, cudaStream_t s);
 size_t ffn_part_bytes(int n_sms);

@@ -14,9 +14,9 @@ MAIN = r"""
 #include <cstdlib>
 #include "pair_rule.cuh"
 int main(int argc, char **argv) {
-  int v[6];
-  for (int i = 0; i < 6; ++i) v[i] = std::atoi(argv[1 + i]);
-  std::puts(xs::pair_rule(v[0], v[1], v[2], v[3], v[4], v[5]) ? "1" : "0");
+  int v[7];
+  for (int i = 0; i < 7; ++i) v[i] = std::atoi(argv[1 + i]);
+  std::puts(xs::pair_rule(v[0], v[1], v[2], v[3] != 0, v[4], v[5], v[6]) ? "1" : "0");
 }
 """
 
@@ -30,8 +30,8 @@ def rule(tmp_path_factory):
     exe = d / "rule"
     subprocess.run(["g++", "-std=c++17", "-I" + CSRC, str(d / "rule.cpp"), "-o", str(exe)], check=True)
 
-    def run(T, N, d, F, here=None, P=76):
-        args = [T * N, N, N if here is None else here, P, d, F]
+    def run(T, N, d, F, here=None, sure=True, P=76):
+        args = [T * N, N, N if here is None else here, int(sure), P, d, F]
         return subprocess.run([str(exe)] + [str(a) for a in args], capture_output=True, text=True,
                               check=True).stdout.strip() == "1"
     return run
@@ -57,4 +57,7 @@ def test_side_that_measured_faster(rule, T, N, d, F, pairs):
 def test_a_rank_counts_its_own_units(rule):
     # 55 experts of 16 blocks fill whole rounds on one GPU; a rank's seven do not.
     assert rule(8, 55, 7168, 2048) and not rule(8, 55, 7168, 2048, here=7)
+    # Plain top-k uses every expert of a rank; of a selection's share the count is a guess.
+    assert rule(16, 256, 7168, 2048, here=32) and rule(8, 256, 7168, 2048, here=32)
+    assert not rule(8, 256, 7168, 2048, here=32, sure=False)
     assert not rule(64, 8, 2048, 256, P=0)   # the kernels cannot run
