@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <cstring>
 
+#include "pair_rule.cuh"
 #include "xs_internal.cuh"
 
 namespace xs {
@@ -99,22 +100,6 @@ RouteArgs route_args(const Plan &pl, void *ws, int B, int N, int k, int budget, 
   a.chunk_marks = at<uint8_t>(ws, pl.chunk_marks);
   a.done = at<int32_t>(ws, pl.done);
   return a;
-}
-
-// At most this many experts can be selected (budgets add to the
-// warm-up sets).
-int max_selected(const RouteArgs &a) {
-  const long long warm = static_cast<long long>(a.B) * a.k0;
-  long long n = a.N;
-  if (a.mode == XS_MODE_BATCH) {
-    n = warm + a.budget;
-  } else if (a.mode == XS_MODE_HIER) {
-    n = warm + static_cast<long long>(a.B / a.T) * a.m_r + a.budget;
-  } else if (a.mode == XS_MODE_GROUP) {
-    const long long rounds = static_cast<long long>(a.m_g) * a.G + a.G - 1;
-    n = warm > rounds ? warm : rounds;
-  }
-  return static_cast<int>(n < a.N ? n : a.N);
 }
 
 }  // namespace
@@ -272,8 +257,8 @@ int xs::forward_impl(const FwdCall &c, FwdStep step) {
   a.zero_words = at<int32_t>(workspace, pl.ffn_cnt);
   a.zero_count = (int)ffn_cnt_words(pl.max_tiles, B, d, F);
   a.n_shared = n_shared;
-  const bool ffn_pairs = ffn_use_pairs(static_cast<long long>(B) * k, max_selected(a), c.mode == XS_MODE_TOPK,
-                                       ep ? c.ep_ranks : 1, d, F);
+  const bool ffn_pairs = ffn_use_pairs(static_cast<long long>(B) * k, selected_at_most(c.mode, B, N, c.budget, a.k0, a.T, a.m_r, a.G, a.m_g),
+                                       c.mode == XS_MODE_TOPK, ep ? c.ep_ranks : 1, d, F);
   if (ffn_pairs) a.tile_tok = kPairTok;
 
   FfnArgs f;

@@ -1,7 +1,28 @@
 // Which batches take the CTA-pair FFN kernels (ffn_pair.cu), host side.
 #pragma once
 
+#include "xshare.h"
+
 namespace xs {
+
+// At most this many experts can be selected (budgets add to the warm-up
+// sets).  Groups are filled in whole rounds, so that without warm-up sets S
+// has m_g G experts; with them the last round may go beyond by G - 1.  (That
+// G - 1 at k0 = 0 made the rule see 47 experts where 40 are selected: N = 64, d =
+// 7168, F = 1024, G = 8, m_g = 5, B = 32 274.7 -> 286.4 us.)
+inline int selected_at_most(int mode, int B, int N, int budget, int k0, int T, int m_r, int G, int m_g) {
+  const long long warm = static_cast<long long>(B) * k0;
+  long long n = N;
+  if (mode == XS_MODE_BATCH) {
+    n = warm + budget;
+  } else if (mode == XS_MODE_HIER) {
+    n = warm + static_cast<long long>(B / T) * m_r + budget;
+  } else if (mode == XS_MODE_GROUP) {
+    const long long rounds = static_cast<long long>(m_g) * G + (k0 > 0 ? G - 1 : 0);
+    n = warm > rounds ? warm : rounds;
+  }
+  return static_cast<int>(n < N ? n : N);
+}
 
 // By T, the pairs per expert that can be selected, and by the time that SMs
 // wait because the pair kernels cut no unit (ffn_tc.cu does):
@@ -35,14 +56,14 @@ namespace xs {
 //   N = 300, d = 640, F = 1920 (21 % in the down phase): T = 15 361.9 | 367.3
 //   N = 256, d = 7168, F = 2048, budget 24, k0 = 1: B = 32 (T = 4.6) 552 | 561,
 //   B = 64 (5.8) 739 | 727, B = 96 (6.4) 858 | 838, B = 128 (6.7) 950 | 938;
-//   groups, B = 256 (8) 772 | 763
+//   groups, B = 256 (8) 772 | 763, B = 32 (5.4) 557 | 565
 constexpr int kPairAllTok = 48;
 constexpr int kPairMinTok = 24;
 constexpr double kPairWait = 70.0;
 constexpr int kPairWaitTok = 32;
 constexpr double kPairWaitAny = 95.0;
 constexpr int kPairFewTok = 12;
-constexpr int kPairWork = 600 * 64;
+constexpr int kPairWork = 650 * 64;
 constexpr double kPairIdle = 0.045;
 
 // `pairs` routed pairs over at most `experts` experts, `here` of them on this
