@@ -1,6 +1,8 @@
 // Which batches take the CTA-pair FFN kernels (ffn_pair.cu), host side.
 #pragma once
 
+#include <initializer_list>
+
 #include "xshare.h"
 
 namespace xs {
@@ -28,8 +30,9 @@ inline int selected_at_most(int mode, int B, int N, int budget, int k0, int T, i
 // wait because the pair kernels cut no unit (ffn_tc.cu does):
 //   - T >= kPairAllTok: always;
 //   - T >= kPairMinTok: unless phases of several rounds of units take more
-//     than kPairWait K steps longer than their work spread evenly over the
-//     pairs would, or (T < kPairWaitTok) all phases more than kPairWaitAny;
+//     than kPairWait K steps (and more than kPairWaitShare of both phases'
+//     work) longer than their work spread evenly over the pairs would, or
+//     (T < kPairWaitTok) phases of one round more than kPairWaitOne;
 //   - T >= kPairFewTok, or T K >= kPairWork (long units hide a unit's fixed
 //     costs): if neither phase idles more than kPairIdle of its time in the
 //     last round of units, or on the missing half of an odd down block.
@@ -49,6 +52,8 @@ inline int selected_at_most(int mode, int B, int N, int budget, int k0, int T, i
 //   68.0 | 61.5; N = 8, d = 7168, F = 256 75.9 | 64.7
 //   T = 48: N = 16, d = 5120, F = 2048 181.6 | 180.3; N = 16, d = 6144, F = 1408
 //   165.8 | 159.1; N = 300, d = 640, F = 1920 406.6 | 413.6; T = 64: 504.2 | 479.2
+//   a small share of the work: d = 7168, F = 2048, 40 experts, T = 25.6 (65 + 8,
+//   5.2 %) 552.7 | 542.5; 64 experts, T = 32 (59 + 14, 3.2 %) 874.3 | 859.4
 // Below T = 24, by the share of idle time:
 //   N = 64, d = 2048, F = 1024 (3.9 %): T = 8 142.1 | 143.5, 12.5 144.4 | 141.1
 //   N = 128, d = 2048, F = 768 (8.9 %): T = 8 201.4 | 203.1, 16 208.1 | 211.4
@@ -60,8 +65,9 @@ inline int selected_at_most(int mode, int B, int N, int budget, int k0, int T, i
 constexpr int kPairAllTok = 48;
 constexpr int kPairMinTok = 24;
 constexpr double kPairWait = 70.0;
+constexpr double kPairWaitShare = 0.055;
 constexpr int kPairWaitTok = 32;
-constexpr double kPairWaitAny = 95.0;
+constexpr double kPairWaitOne = 95.0;
 constexpr int kPairFewTok = 12;
 constexpr int kPairWork = 650 * 64;
 constexpr double kPairIdle = 0.045;
@@ -91,9 +97,10 @@ inline bool pair_rule(long long pairs, int experts, int here, bool sure, int P, 
   };
   const Phase gate_up = phase(F / 128, F / 128.0, d), down = phase((d + 255) / 256, d / 256.0, F);
   if (tokens(kPairMinTok)) {
-    const double several =
-        (gate_up.rounds > 1 ? gate_up.waited() : 0.0) + (down.rounds > 1 ? down.waited() : 0.0);
-    return several <= kPairWait && (tokens(kPairWaitTok) || gate_up.waited() + down.waited() <= kPairWaitAny);
+    double several = 0.0, one = 0.0;
+    for (const Phase *p : {&gate_up, &down}) (p->rounds > 1 ? several : one) += p->waited();
+    const double share = kPairWaitShare * (gate_up.even * gate_up.steps + down.even * down.steps);
+    return several <= (share > kPairWait ? share : kPairWait) && (tokens(kPairWaitTok) || one <= kPairWaitOne);
   }
   if (!sure) return false;
   if (!tokens(kPairFewTok) && pairs * d < static_cast<long long>(kPairWork) * experts) return false;

@@ -44,11 +44,11 @@ cudaError_t launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, size_t 
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
-// Both FFN paths round alike: a correctly rounded division.  The pairs' gate/up
-// epilogue runs under the next unit's MMAs; the fast division (2 ulp) saved it
-// 0.7 to 1 % of the layer at d = 2048, F = 1024, B = 2048 and 8192 (249.6
-// instead of 251.5 us, 711 instead of 717) and less elsewhere, and changed y by
-// 1e-4 when a batch took the pairs.
+// Both FFN paths round alike: a correctly rounded division.  The fast one (2
+// ulp) saved the pairs' gate/up epilogue up to 4 us, where a phase's last units
+// weigh most (layer forward, fast -> this: d = 2048, F = 1024, 16 experts, B = 256
+// 73.8 -> 76.6 us, B = 8192 711 -> 717), and changed y by 1e-4 when a batch took
+// the pairs.
 __device__ __forceinline__ float silu(float g) { return g / (1.f + expf(-g)); }
 
 // Drops the 128-byte line at p (aligned) from L2 without writing it back.

@@ -57,6 +57,8 @@ def rule(exe):
     (24, 300, 640, 1920, False), (32, 300, 640, 1920, False), (64, 300, 640, 1920, True),
     (24, 16, 6144, 1408, False), (32, 16, 6144, 1408, False), (48, 16, 6144, 1408, True),
     (24, 16, 7168, 2048, False), (64, 16, 7168, 2048, True),
+    # As long a wait, but of a wide layer's work.
+    (25, 40, 7168, 2048, True), (32, 64, 7168, 2048, True),
     # One round of long units on few SMs: a loss at 24 tokens, a gain at 32.
     (24, 4, 7168, 256, False), (32, 4, 7168, 256, True), (24, 8, 7168, 256, True),
     # Few or narrow experts that gain.
